@@ -31,6 +31,20 @@ __device__ __forceinline__ uint32_t smid()
     return r;
 }
 
+// True in exactly one lane of a converged warp.  A branch on this predicate, unlike one on the lane index, lets the
+// compiler treat the operands of single-thread instructions (tcgen05.mma, tcgen05.commit, bulk tensor copies) as
+// warp-uniform.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t pred;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.b32 %0, 1, 0, p;\n\t}"
+        : "=r"(pred));
+    return pred != 0;
+}
+
 // ------------------------------------------------------------------ programmatic dependent launch
 
 // Block until the grids this launch depends on have completed and their memory is visible

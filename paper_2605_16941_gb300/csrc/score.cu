@@ -39,6 +39,15 @@
 //           only, the MMA issuer: 4 x (M256 Nbn K16) per stage and tile,
 //           committing stage release and accumulator-ready to both CTAs
 //           (multicast);
+//           Both of these roles run in one thread of their warp, chosen by
+//           elect.sync: behind a branch on the lane index the compiler cannot
+//           know that the operands of tcgen05.mma, tcgen05.commit and the
+//           copies are warp-uniform, and issuing a K slice's MMAs then took
+//           longer than the MMAs themselves.  Branch on the lane index and a
+//           shuffle per wait, then elect.sync (us per step, 20-step regions at
+//           full clock; d = 4096, V = 126464): N = 64 168 -> 156, N = 256
+//           179 -> 166, N = 2048 1092 -> 1070; d = 1024, V = 64000, N = 2048
+//           247 -> 201;
 //   warps 2-5 epilogue (both CTAs): one thread per row (TMEM lane); online
 //           softmax over a tile's columns, then release of the accumulator to
 //           the leader's MMA warp (8 arrivals per accumulator use).
@@ -274,41 +283,34 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
         // nothing to do: the status word reports the failed allocation check
     } else if (warp == 0) {
         // ------------------------------------------------------------ TMA producer (both CTAs)
-        const int half_bn = a.bn >> 1;  // W rows each CTA stages per tile
-        // W map coordinates of (K slice kb, vocabulary row v): (64 kb, v) in row-major W, (0, kb V + v) in the
-        // panel copy
-        auto w_x = [&](int kb) { return a.w_panels ? 0 : kb * kBK; };
-        auto w_y = [&](int kb, int v) { return a.w_panels ? kb * a.V + v : v; };
-        if (lane == 0 && grp < a.n_mb)
-            for (int kb = 0; kb < min(a.n_kb, kPrefetchSlices); ++kb)
-                ptx::tma_prefetch_2d(&tmW, w_x(kb), w_y(kb, col * a.bn + (int)rank * half_bn));
-        ptx::grid_dep_wait();
-        const uint64_t pol_h = ptx::policy_evict_last();    // H is re-read for every item
-        const uint64_t pol_w = ptx::policy_evict_normal();  // W is shared by the row-block groups
-        int stage = 0;
-        uint32_t phase = 0;
-        int32_t issued_parity[kMaxStages];
-        for (int s = 0; s < kMaxStages; ++s)
-            issued_parity[s] = -1;
-        bool aborted = false;
-        bool first = true;
-        for (int mb = grp; mb < a.n_mb && !aborted; mb += mb_step) {
-            const int mb2 = mb + a.n_groups;  // partner row block of a row-pair sweep
-            const bool rows2 = kTwo && mb2 < a.n_mb;
-            for (int vt = col; vt < a.n_vt && !aborted; vt += rows2 ? a.G : vstep) {
-                const bool two = kTwo && (rows2 || vt + a.G < a.n_vt);
-                // both CTAs' copies: H, the tile's W, and the partner block's H or the second tile's W
-                const uint32_t stage_tx = 2u * (kStageBytesA + wb + (rows2 ? kStageBytesA : (two ? wb : 0u)));
-                for (int kb = 0; kb < a.n_kb; ++kb) {
-                    int ok = 1;
-                    if (lane == 0)
-                        ok = wait_bounded(empty(stage), phase ^ 1u, &bars->abort);
-                    ok = __shfl_sync(0xffffffffu, ok, 0);
-                    if (!ok) {
-                        aborted = true;
-                        break;
-                    }
-                    if (lane == 0) {
+        if (ptx::elect_one()) {
+            const int half_bn = a.bn >> 1;  // W rows each CTA stages per tile
+            // W map coordinates of (K slice kb, vocabulary row v): (64 kb, v) in row-major W, (0, kb V + v) in the
+            // panel copy
+            auto w_x = [&](int kb) { return a.w_panels ? 0 : kb * kBK; };
+            auto w_y = [&](int kb, int v) { return a.w_panels ? kb * a.V + v : v; };
+            if (grp < a.n_mb)
+                for (int kb = 0; kb < min(a.n_kb, kPrefetchSlices); ++kb)
+                    ptx::tma_prefetch_2d(&tmW, w_x(kb), w_y(kb, col * a.bn + (int)rank * half_bn));
+            ptx::grid_dep_wait();
+            const uint64_t pol_h = ptx::policy_evict_last();    // H is re-read for every item
+            const uint64_t pol_w = ptx::policy_evict_normal();  // W is shared by the row-block groups
+            int stage = 0;
+            uint32_t phase = 0;
+            int64_t issued = 0;  // stages filled so far
+            bool aborted = false;
+            for (int mb = grp; mb < a.n_mb && !aborted; mb += mb_step) {
+                const int mb2 = mb + a.n_groups;  // partner row block of a row-pair sweep
+                const bool rows2 = kTwo && mb2 < a.n_mb;
+                for (int vt = col; vt < a.n_vt && !aborted; vt += rows2 ? a.G : vstep) {
+                    const bool two = kTwo && (rows2 || vt + a.G < a.n_vt);
+                    // both CTAs' copies: H, the tile's W, and the partner block's H or the second tile's W
+                    const uint32_t stage_tx = 2u * (kStageBytesA + wb + (rows2 ? kStageBytesA : (two ? wb : 0u)));
+                    for (int kb = 0; kb < a.n_kb; ++kb) {
+                        if (!wait_bounded(empty(stage), phase ^ 1u, &bars->abort)) {
+                            aborted = true;
+                            break;
+                        }
                         const uint32_t bar = ptx::mapa(full(stage), 0);  // the leader's stage barrier
                         if (leader)
                             ptx::mbar_arrive_expect_tx(full(stage), stage_tx);
@@ -321,29 +323,26 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
                         else if (two)
                             ptx::tma_load_2d_pair(sB(stage, 1), &tmW, bar, w_x(kb),
                                                   w_y(kb, (vt + a.G) * a.bn + (int)rank * half_bn), pol_w);
-                        if (tl && first)
+                        if (tl && issued == 0)
                             tl[2] = ptx::globaltimer_ns();
-                        first = false;
-                    }
-                    __syncwarp();
-                    issued_parity[stage] = (int32_t)phase;
-                    if (++stage == S) {
-                        stage = 0;
-                        phase ^= 1u;
+                        ++issued;
+                        if (++stage == S) {
+                            stage = 0;
+                            phase ^= 1u;
+                        }
                     }
                 }
             }
-        }
-        if (aborted && leader && lane == 0) {
-            // Let every copy already issued (by either CTA) land before the pair's shared memory goes away.
-            for (int s = 0; s < S; ++s)
-                if (issued_parity[s] >= 0)
-                    wait_drain(full(s), (uint32_t)issued_parity[s]);
+            if (aborted && leader) {
+                // Let every copy already issued (by either CTA) land before the pair's shared memory goes away.
+                for (int s = 0; s < S && s < issued; ++s)
+                    wait_drain(full(s), (uint32_t)((issued - 1 - s) / S) & 1u);
+            }
         }
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer (leader)
-        if (leader) {
+        if (leader && ptx::elect_one()) {
             const uint32_t idesc = ptx::idesc_bf16_f32(kPairM, (uint32_t)a.bn);
             int tiles = 0;
             int stage = 0;
@@ -351,12 +350,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
             int item = 0;  // items issued so far
             bool aborted = false;
             auto wait_acc_free = [&](int i, uint32_t uses) -> bool {  // the epilogue has read use uses-1 of acc i
-                int ok = 1;
-                if (lane == 0)
-                    ok = wait_bounded<true>(tempty(i), (uses & 1u) ^ 1u, &bars->abort);
-                ok = __shfl_sync(0xffffffffu, ok, 0);
+                const bool ok = wait_bounded<true>(tempty(i), (uses & 1u) ^ 1u, &bars->abort);
                 ptx::tc_fence_after();
-                return ok != 0;
+                return ok;
             };
             auto issue = [&](int acc, uint32_t a_smem, uint32_t b_smem, int kb) {  // 4 x K16 from one stage
                 const uint64_t da = ptx::sdesc_kmajor_sw128(a_smem);
@@ -370,10 +366,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
                 // accumulator 1 of a pass: the partner block's H (third slot) x the tile's W, or this block's
                 // H x the second tile's W (third slot)
                 auto issue1 = [&](int s, int kb) {
-                    if (rows2)
-                        issue(1, sB(s, 1), sB(s, 0), kb);
-                    else
-                        issue(1, sA(s), sB(s, 1), kb);
+                    issue(1, rows2 ? sB(s, 1) : sA(s), rows2 ? sB(s, 0) : sB(s, 1), kb);
                 };
                 for (int vt = col; vt < a.n_vt && !aborted; vt += rows2 ? a.G : vstep, ++item) {
                     const bool two = kTwo && (rows2 || vt + a.G < a.n_vt);
@@ -388,36 +381,30 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
                     const int defer = two ? min(S, a.n_kb) : 0;  // stages whose second-accumulator MMAs wait
                     const int s0 = stage;
                     for (int kb = 0; kb < a.n_kb; ++kb) {
-                        int ok = 1;
-                        if (lane == 0)
-                            ok = wait_bounded(full(stage), phase, &bars->abort);
-                        ok = __shfl_sync(0xffffffffu, ok, 0);
-                        if (!ok) {
+                        if (!wait_bounded(full(stage), phase, &bars->abort)) {
                             aborted = true;
                             break;
                         }
-                        ptx::tc_fence_after();
-                        if (lane == 0)
-                            issue(acc0, sA(stage), sB(stage, 0), kb);
+                        issue(acc0, sA(stage), sB(stage, 0), kb);
                         if (kb < defer) {
                             if (kb == defer - 1) {  // the second accumulator is needed now
                                 if (!wait_acc_free(1, (uint32_t)item)) {
                                     aborted = true;
                                     break;
                                 }
-                                if (lane == 0)
-                                    for (int j = 0; j < defer; ++j) {
-                                        const int sj = (s0 + j) % S;
-                                        issue1(sj, j);
-                                        ptx::mma_commit_pair_multicast(empty(sj), kBothCtas);
-                                    }
+                                int sj = s0;
+                                for (int j = 0; j < defer; ++j) {
+                                    issue1(sj, j);
+                                    ptx::mma_commit_pair_multicast(empty(sj), kBothCtas);
+                                    if (++sj == S)
+                                        sj = 0;
+                                }
                             }
-                        } else if (lane == 0) {
+                        } else {
                             if (two)
                                 issue1(stage, kb);
                             ptx::mma_commit_pair_multicast(empty(stage), kBothCtas);
                         }
-                        __syncwarp();
                         if (++stage == S) {
                             stage = 0;
                             phase ^= 1u;
@@ -425,26 +412,21 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
                     }
                     if (aborted)
                         break;
-                    if (lane == 0) {
-                        ptx::mma_commit_pair_multicast(tfull(acc0), kBothCtas);
-                        if (kTwo)  // the epilogue waits for both accumulators of every pass
-                            ptx::mma_commit_pair_multicast(tfull(1), kBothCtas);
-                    }
-                    __syncwarp();
+                    ptx::mma_commit_pair_multicast(tfull(acc0), kBothCtas);
+                    if (kTwo)  // the epilogue waits for both accumulators of every pass
+                        ptx::mma_commit_pair_multicast(tfull(1), kBothCtas);
                     tiles += two ? 2 : 1;
                 }
             }
             // No MMA may still be writing either CTA's TMEM when it is released.
-            if (lane == 0) {
-                ptx::mma_commit_pair(mma_done);
-                wait_drain(mma_done, 0);
-                if (tl) {
-                    tl[4] = ptx::globaltimer_ns();
-                    tl[7] = (uint64_t)ptx::smid() << 32 | (uint32_t)tiles;
-                }
+            ptx::mma_commit_pair(mma_done);
+            wait_drain(mma_done, 0);
+            if (tl) {
+                tl[4] = ptx::globaltimer_ns();
+                tl[7] = (uint64_t)ptx::smid() << 32 | (uint32_t)tiles;
             }
-            __syncwarp();
         }
+        __syncwarp();
     } else {
         // ------------------------------------------------------------ epilogue (warps 2..5, both CTAs)
         const int q = warp & 3;  // this warp may only read TMEM lanes [32q, 32q + 32)
