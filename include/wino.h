@@ -365,8 +365,10 @@ WINO_API int wino_timeline_begin(uint64_t *buf, int64_t n_launches, int64_t ctas
 WINO_API int wino_timeline_end(int64_t *launches);
 
 /*
- * How a score launch of N rows over V entries is split on the current device
- * (diagnostics; the paper has no counterpart): plan (host int32[8]) receives
+ * How the row-block score kernel splits a launch of N rows over V entries on
+ * the current device (diagnostics; the paper has no counterpart).  Row counts
+ * that do not fill 256-row blocks mostly run on the vocabulary-major kernel
+ * instead, whose split this call does not describe.  plan (host int32[8]) receives
  * the tile width bn, the vocabulary tiles n_vt = ceil(V / bn), the 256-row
  * blocks n_mb, the row-block groups, the CTA pairs per group G (= records per
  * row), the grid size in CTAs, 1 if the kernel works in passes (each staged

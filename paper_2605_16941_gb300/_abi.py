@@ -300,14 +300,14 @@ def wino_profile_end() -> tuple[float, int]:
 
 
 def wino_score_plan(N: int, d: int, V: int) -> dict:
-    """The score kernel's work split for N rows over V entries on the current device."""
+    """The row-block score kernel's work split for N rows over V entries on the current device."""
     out = (C.c_int32 * 8)()
     _check(lib().wino_score_plan(int(N), int(d), int(V), out), "wino_score_plan")
     return dict(zip(("bn", "n_vt", "n_mb", "n_groups", "G", "ctas", "two", "stages"), list(out)))
 
 
 def wino_score_plan_host(N: int, d: int, V: int, sm_count: int = 152, max_pairs: int = 76) -> dict:
-    """The score kernel's work split for a device with sm_count SMs and max_pairs resident pairs (no device)."""
+    """The row-block score kernel's work split for a device with sm_count SMs and max_pairs resident pairs (no device)."""
     out = (C.c_int32 * 10)()
     _check(lib().wino_score_plan_host(int(N), int(d), int(V), int(sm_count), int(max_pairs), out),
            "wino_score_plan_host")

@@ -34,50 +34,15 @@
 // is applied in place in one pass after a CTA-wide reduction.  With
 // WINO_OPT_FREEZE_FINISHED a sequence whose block already has no MASK is left
 // as it is (its own loop, Sec. 4.2.3, has ended).
+#include "fold.cuh"
 #include "internal.h"
 #include "ptx.cuh"
 
 namespace wino {
 namespace {
 
-constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr int kFinishRows = 8;  // rows (warps) per finish CTA; also the CTA size of the Eq. 4 kernels
-
-// Fold (m2, s2, i2) into (m, s, i): the larger max wins, the smaller index on equal maxima.
-__device__ __forceinline__ void combine(float &m, float &s, int32_t &i, float m2, float s2, int32_t i2)
-{
-    const float M = fmaxf(m, m2);
-    const float a = (m == -INFINITY) ? 0.f : s * ptx::ex2((m - M) * kLog2e);
-    const float b = (m2 == -INFINITY) ? 0.f : s2 * ptx::ex2((m2 - M) * kLog2e);
-    if (m2 > m || (m2 == m && i2 < i))
-        i = i2;
-    m = M;
-    s = a + b;
-}
-
-// As combine, also folding u = sum exp(l - m) (l - m) log2(e) (rescaled to the new max like s).
-__device__ __forceinline__ void combine_u(float &m, float &s, float &u, int32_t &i, float m2, float s2, float u2,
-                                          int32_t i2)
-{
-    const float M = fmaxf(m, m2);
-    float a = 0.f, b = 0.f, ua = 0.f, ub = 0.f;
-    if (m != -INFINITY) {
-        const float al = ptx::ex2((m - M) * kLog2e);
-        a = s * al;
-        ua = al * fmaf((m - M) * kLog2e, s, u);
-    }
-    if (m2 != -INFINITY) {
-        const float bl = ptx::ex2((m2 - M) * kLog2e);
-        b = s2 * bl;
-        ub = bl * fmaf((m2 - M) * kLog2e, s2, u2);
-    }
-    if (m2 > m || (m2 == m && i2 < i))
-        i = i2;
-    m = M;
-    s = a + b;
-    u = ua + ub;
-}
 
 // Block-wide reduction scratch for eq4_block.
 struct Eq4Smem {

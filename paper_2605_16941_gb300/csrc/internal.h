@@ -42,6 +42,17 @@ constexpr uint32_t kTmemCols = 2 * kBN;  // two 256-column fp32 accumulators: al
 // W bytes one CTA stages per K slice of a tile of width bn (bn/2 rows of 128 B; a multiple of 1 KB).
 __host__ __device__ constexpr uint32_t stage_bytes_w(int bn) { return (uint32_t)(bn / 2) * kBK * 2; }
 
+// Vocabulary-major score kernel (score_vmajor.cu): the vocabulary on the M side of the MMA, hw rows of H (at most
+// 256) per accumulator on the N side, one or two accumulators per vocabulary tile.  Per K slice a CTA stages bn/2 W
+// rows (a 128-row slot) and half of the tile's rows of H.
+constexpr int kVmMaxStages = 12;
+constexpr int kVmMaxSlots = 4;    // accumulators in TMEM
+constexpr int kVmMaxRows = 512;   // rows of H per group of pairs
+constexpr uint32_t kVmStageBytesW = 128u * kBK * 2;
+constexpr uint32_t kVmBarrierBytes = 512;
+constexpr uint32_t kVmSmemOverhead = 1024 /* ring alignment slack */ + kVmBarrierBytes + 8 * 4096 /* transposes */;
+constexpr uint32_t kVmRingCapacity = kScoreSmemMax - kVmSmemOverhead;
+
 constexpr int kMaxBlkLen = 1024;
 
 // Where a scored row's target token comes from.
@@ -111,9 +122,10 @@ struct ScoreArgs {
     int32_t stages;            // ring stages, 2..kMaxStages
     uint32_t stage_bytes;      // 16 KB + stage_bytes_w(bn) + a pass's third slot (W, or 16 KB of H)
     int32_t n_groups, G;
+    int32_t hw[2], slots;  // vocabulary-major kernel only: rows of each accumulator of a tile, accumulators in TMEM
     TargetSource ts;
-    float4 *part;       // [N][G]
-    float *part_u;      // [N][G], entropy variant only: sum of exp(l - m) * (l - m) * log2(e) over the pair's tiles
+    float4 *part;       // [N][records per row: G, or 2 G (one per CTA) from the vocabulary-major kernel]
+    float *part_u;      // the same shape, entropy variant only: sum of exp(l - m) * (l - m) * log2(e) over the pair's tiles
     StatusWords *status;
     int32_t *tickets;   // [n_tickets], cleared here for the finish kernel
     int32_t n_tickets;
@@ -125,7 +137,7 @@ struct FinishArgs {
     const float4 *part;
     const float *part_u;  // with entropy != nullptr
     float *entropy;       // optional: H(p) = -sum_v p_v log p_v per row
-    int32_t G, N, V;
+    int32_t G, N, V;      // G: records per row
     TargetSource ts;
     StatusWords *status;  // read; WINO_ERR_ARG added when an active-sequence list entry is out of range
     int32_t *argmax;
@@ -146,8 +158,20 @@ struct ScoreSchedule {
     int32_t bn, n_vt, n_groups, G;
     int32_t two, stages;
     uint32_t stage_bytes;
+    int64_t cost;  // accumulator columns on the busiest pair, overheads included
 };
 ScoreSchedule score_schedule(int32_t n_mb, int64_t V, int max_units, int32_t records_cap);
+
+// Work split of a vocabulary-major launch.  score_vmajor_schedule returns whether the vocabulary-major kernel takes
+// the launch (its rule stands in score_vmajor.cu); `rows` is the split score.cu would use.
+struct VmSchedule {
+    int32_t bn, n_vt, n_groups, G;
+    int32_t hw[2], slots, stages;
+    uint32_t stage_bytes;
+    int64_t cost;
+};
+bool score_vmajor_schedule(int64_t N, int64_t d, int64_t V, int max_units, int32_t records_cap,
+                           const ScoreSchedule &rows, VmSchedule *out);
 
 // Records per row the workspace reserves for a vocabulary of V entries: one per tile at the narrowest
 // width, at most kMaxRecordsPerRow.
@@ -163,6 +187,13 @@ int score_max_pairs();
 // entropy: also accumulate part_u (the variant used when wino_score_rows is asked for H(p)).
 cudaError_t launch_score(const CUtensorMap &tmH, const CUtensorMap &tmW, const ScoreArgs &a, bool entropy,
                          cudaStream_t stream);
+
+cudaError_t launch_score_vmajor(const CUtensorMap &tmH, const CUtensorMap &tmW, const ScoreArgs &a, bool entropy,
+                                cudaStream_t stream);
+
+// Launch configuration of a score kernel: clusters of two CTAs, programmatic dependent launch.
+cudaLaunchConfig_t score_launch_config(unsigned grid, unsigned threads, uint32_t smem, cudaStream_t stream,
+                                       cudaLaunchAttribute (&attr)[2]);
 
 cudaError_t launch_finish(const FinishArgs &a, cudaStream_t stream);
 

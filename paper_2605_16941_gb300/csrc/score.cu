@@ -12,6 +12,9 @@
 // pair's vocabulary tiles of that row block.  One partial record per
 // (row, pair) goes to the workspace; finish.cu merges them.
 //
+// Row counts that leave much of their 256-row blocks empty, and a few others, go to the vocabulary-major kernel
+// instead (score_vmajor.cu; the rule is score_vmajor_schedule).
+//
 // Two modes (ScoreArgs::two, chosen per launch by score_schedule):
 //   single tiles, for shapes bound by the W stream from HBM (one 256-row
 //     block): the two accumulators alternate between consecutive tiles, so
@@ -65,6 +68,7 @@
 // [7] = SM id << 32 | tiles of the pair.
 #include <mutex>
 
+#include "fold.cuh"
 #include "internal.h"
 #include "ptx.cuh"
 #include "wait.cuh"
@@ -72,7 +76,6 @@
 namespace wino {
 namespace {
 
-constexpr float kLog2e = 1.4426950408889634f;
 constexpr uint16_t kBothCtas = 0x3;
 constexpr int kPrefetchSlices = 4;   // K slices of the first W tile prefetched into L2 before the grid wait
 constexpr int kTmemLoadsPerWait = 1;  // 32-column TMEM loads in flight per tcgen05.wait::ld in the epilogue (2 measured slower)
@@ -87,86 +90,6 @@ struct alignas(8) Barriers {
     int32_t abort;
 };
 static_assert(sizeof(Barriers) <= 256, "barrier block must fit its reserve");
-
-// Running softmax state of one row (one thread), across all of a pair's tiles of that row.
-struct RowState {
-    float m, s0, s1, s2, s3, tlog;
-    float u0, u1, u2, u3;  // entropy variant: sum of exp(l - m) (l - m) log2(e)
-    int32_t am;
-};
-
-// Fold 32 consecutive logits x (columns v .. v + 31; those at or past cvalid are not logits) into the row
-// state: online max with rescaling, four partial sums of 2^((l - m) log2 e), argmax (an earlier column
-// keeps it on ties), and the target's logit when it lies among them.
-template <bool kEntropy>
-__device__ __forceinline__ void fold32(RowState &r, float (&x)[32], int v, int cvalid, int tgt)
-{
-    if (cvalid < 32) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-            if (j >= cvalid)
-                x[j] = -INFINITY;  // past V (TMA zero fill) or past the tile (another tile's columns)
-    }
-    float cm = x[0];
-#pragma unroll
-    for (int j = 1; j < 32; ++j)
-        cm = fmaxf(cm, x[j]);
-    if (cm > r.m) {  // strict: an earlier column keeps the argmax on ties
-        int j0 = 31;
-#pragma unroll
-        for (int j = 31; j >= 0; --j)
-            if (x[j] == cm)
-                j0 = j;
-        r.am = v + j0;
-        const float scale = ptx::ex2((r.m - cm) * kLog2e);
-        if (kEntropy && r.m != -INFINITY) {  // u' = scale * (u + (m - cm) log2(e) * s)
-            const float dl = (r.m - cm) * kLog2e;
-            r.u0 = scale * fmaf(dl, r.s0, r.u0);
-            r.u1 = scale * fmaf(dl, r.s1, r.u1);
-            r.u2 = scale * fmaf(dl, r.s2, r.u2);
-            r.u3 = scale * fmaf(dl, r.s3, r.u3);
-        }
-        r.s0 *= scale;
-        r.s1 *= scale;
-        r.s2 *= scale;
-        r.s3 *= scale;
-        r.m = cm;
-    }
-    const float mb2 = r.m * kLog2e;
-    if (!kEntropy) {
-#pragma unroll
-        for (int j = 0; j < 32; j += 4) {
-            r.s0 += ptx::ex2(fmaf(x[j + 0], kLog2e, -mb2));
-            r.s1 += ptx::ex2(fmaf(x[j + 1], kLog2e, -mb2));
-            r.s2 += ptx::ex2(fmaf(x[j + 2], kLog2e, -mb2));
-            r.s3 += ptx::ex2(fmaf(x[j + 3], kLog2e, -mb2));
-        }
-    } else {
-        // t = (l - m) log2(e), kept finite (masked columns are -inf; 2^-200 is 0 in fp32 anyway)
-#pragma unroll
-        for (int j = 0; j < 32; j += 4) {
-            const float t0 = fmaxf(fmaf(x[j + 0], kLog2e, -mb2), -200.f);
-            const float t1 = fmaxf(fmaf(x[j + 1], kLog2e, -mb2), -200.f);
-            const float t2 = fmaxf(fmaf(x[j + 2], kLog2e, -mb2), -200.f);
-            const float t3 = fmaxf(fmaf(x[j + 3], kLog2e, -mb2), -200.f);
-            const float e0 = ptx::ex2(t0), e1 = ptx::ex2(t1), e2 = ptx::ex2(t2), e3 = ptx::ex2(t3);
-            r.s0 += e0;
-            r.s1 += e1;
-            r.s2 += e2;
-            r.s3 += e3;
-            r.u0 = fmaf(e0, t0, r.u0);
-            r.u1 = fmaf(e1, t1, r.u1);
-            r.u2 = fmaf(e2, t2, r.u2);
-            r.u3 = fmaf(e3, t3, r.u3);
-        }
-    }
-    const int tj = tgt - v;
-    if ((unsigned)tj < 32u) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-            r.tlog = (j == tj) ? x[j] : r.tlog;
-    }
-}
 
 // Fold the nvalid first columns of one accumulator (this warp's 32 TMEM lanes from tbase), vocabulary
 // ids v0 ..; kTmemLoadsPerWait 32-column loads in flight per wait.
@@ -546,7 +469,7 @@ ScoreSchedule score_schedule(int32_t n_mb, int64_t V, int max_units, int32_t rec
     constexpr int64_t kTileOverheadCols = 16;  // single tiles: H re-staged per tile, in columns
     constexpr int64_t kPassOverheadCols = 32;  // passes: the epilogue the next pass partly waits for
     const int32_t two = n_mb >= kPassMinRowBlocks ? 1 : 0;
-    ScoreSchedule best{kBN, (int32_t)((V + kBN - 1) / kBN), 1, 1, two, 2, 0};
+    ScoreSchedule best{kBN, (int32_t)((V + kBN - 1) / kBN), 1, 1, two, 2, 0, 0};
     int64_t best_cost = -1;
     const int32_t top = n_mb < max_units ? n_mb : max_units;
     for (int32_t bn = kBN; bn >= kMinBN; bn -= 16) {
@@ -570,6 +493,7 @@ ScoreSchedule score_schedule(int32_t n_mb, int64_t V, int max_units, int32_t rec
             }
         }
     }
+    best.cost = best_cost;
     // A pass stage has a third slot: the second tile's W, or in a row-pair sweep (a group with more than
     // one row block) the partner block's H.
     const uint32_t wb = stage_bytes_w(best.bn);
@@ -580,13 +504,12 @@ ScoreSchedule score_schedule(int32_t n_mb, int64_t V, int max_units, int32_t rec
     return best;
 }
 
-namespace {
-
-cudaLaunchConfig_t score_config(unsigned grid, uint32_t smem, cudaStream_t stream, cudaLaunchAttribute (&attr)[2])
+cudaLaunchConfig_t score_launch_config(unsigned grid, unsigned threads, uint32_t smem, cudaStream_t stream,
+                                       cudaLaunchAttribute (&attr)[2])
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(kScoreThreads);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -599,6 +522,8 @@ cudaLaunchConfig_t score_config(unsigned grid, uint32_t smem, cudaStream_t strea
     cfg.numAttrs = 2;
     return cfg;
 }
+
+namespace {
 
 // Per-device one-time set-up: shared-memory opt-in and the number of co-resident pairs.
 int configure_device()
@@ -618,7 +543,7 @@ int configure_device()
                 return -1;
         cudaLaunchAttribute attr[2];
         // Any launch's shared memory exceeds half an SM's, so one CTA per SM whatever the ring size.
-        cudaLaunchConfig_t cfg = score_config(2, kScoreSmemMax, nullptr, attr);
+        cudaLaunchConfig_t cfg = score_launch_config(2, kScoreThreads, kScoreSmemMax, nullptr, attr);
         cfg.numAttrs = 1;  // the cluster shape is what matters for the occupancy query
         int clusters = 0;
         if (cudaOccupancyMaxActiveClusters(&clusters, score_kernel<false, true>, &cfg) != cudaSuccess || clusters < 1)
@@ -646,8 +571,8 @@ cudaError_t launch_score(const CUtensorMap &tmH, const CUtensorMap &tmW, const S
         a.stage_bytes % 1024u != 0 || (uint64_t)a.stages * a.stage_bytes > kRingCapacity)
         return cudaErrorInvalidValue;
     cudaLaunchAttribute attr[2];
-    cudaLaunchConfig_t cfg = score_config((unsigned)(2 * a.n_groups * a.G),
-                                          kSmemOverhead + (uint32_t)a.stages * a.stage_bytes, stream, attr);
+    cudaLaunchConfig_t cfg = score_launch_config((unsigned)(2 * a.n_groups * a.G), kScoreThreads,
+                                                 kSmemOverhead + (uint32_t)a.stages * a.stage_bytes, stream, attr);
     if (entropy)
         return a.two ? cudaLaunchKernelEx(&cfg, score_kernel<true, true>, tmH, tmW, a)
                      : cudaLaunchKernelEx(&cfg, score_kernel<true, false>, tmH, tmW, a);

@@ -233,10 +233,20 @@ int score_and_finish(const uint16_t *H, const uint16_t *W, bool w_panels, int64_
     if (max_pairs < 1)
         return WINO_ERR_CUDA;
     const int32_t n_mb = (int32_t)((N + kPairM - 1) / kPairM);
-    const ScoreSchedule sch =
-        score_schedule(n_mb, V, std::min(max_pairs, info.sm_count / 2), (int32_t)records_per_row(V));
+    const int units = std::min(max_pairs, info.sm_count / 2);
+    ScoreSchedule sch = score_schedule(n_mb, V, units, (int32_t)records_per_row(V));
+    VmSchedule vm{};
+    const bool vmajor = score_vmajor_schedule(N, d, V, units, (int32_t)records_per_row(V), sch, &vm);
+    if (vmajor) {
+        sch.bn = vm.bn;
+        sch.n_vt = vm.n_vt;
+        sch.n_groups = vm.n_groups;
+        sch.G = vm.G;
+        sch.stages = vm.stages;
+        sch.stage_bytes = vm.stage_bytes;
+    }
     CUtensorMap tmH, tmW;
-    if ((rc = tensor_map(H, N, d, kBM, &tmH)) != WINO_OK)
+    if ((rc = tensor_map(H, N, d, vmajor ? (vm.hw[0] + vm.hw[1]) / 2 : kBM, &tmH)) != WINO_OK)
         return rc;
     // one 16-byte-aligned map row per (K slice, vocabulary row) of the panel copy
     if ((rc = w_panels ? tensor_map(W, d / kBK * V, kBK, sch.bn / 2, &tmW) : tensor_map(W, V, d, sch.bn / 2, &tmW)) !=
@@ -256,6 +266,9 @@ int score_and_finish(const uint16_t *H, const uint16_t *W, bool w_panels, int64_
     a.stage_bytes = sch.stage_bytes;
     a.n_groups = sch.n_groups;
     a.G = sch.G;
+    a.hw[0] = vm.hw[0];
+    a.hw[1] = vm.hw[1];
+    a.slots = vm.slots;
     a.ts = ts;
     a.part = reinterpret_cast<float4 *>(w8 + L.part);
     a.part_u = entropy ? reinterpret_cast<float *>(w8 + L.part_u) : nullptr;
@@ -265,14 +278,15 @@ int score_and_finish(const uint16_t *H, const uint16_t *W, bool w_panels, int64_
     a.timeline = timeline_slot((unsigned)(2 * a.n_groups * a.G));
     a.w_panels = w_panels ? 1 : 0;
     prof_record(0, stream);
-    if (launch_score(tmH, tmW, a, entropy != nullptr, stream) != cudaSuccess)
+    if ((vmajor ? launch_score_vmajor(tmH, tmW, a, entropy != nullptr, stream)
+                : launch_score(tmH, tmW, a, entropy != nullptr, stream)) != cudaSuccess)
         return WINO_ERR_CUDA;
     prof_record(1, stream);
     FinishArgs f{};
     f.part = a.part;
     f.part_u = a.part_u;
     f.entropy = entropy;
-    f.G = a.G;
+    f.G = vmajor ? 2 * a.G : a.G;  // one record per CTA of a pair from the vocabulary-major kernel
     f.N = a.N;
     f.V = a.V;
     f.ts = ts;
