@@ -32,7 +32,10 @@ constexpr int kBN = 256;     // largest tile width (UMMA N); TMEM column stride 
 constexpr int kMinBN = 128;  // narrowest tile width the schedule uses
 constexpr int kBK = 64;
 constexpr int kMaxStages = 7;
-constexpr int kScoreThreads = 192;  // warp 0 TMA, warp 1 TMEM + MMA, warps 2-5 epilogue
+constexpr int kEpiPerQuarter = 2;  // epilogue warps per TMEM lane quarter
+constexpr int kEpiWarps = 4 * kEpiPerQuarter;
+constexpr int kScoreThreads = 64 + 32 * kEpiWarps;  // warp 0 TMA, warp 1 TMEM + MMA, then the epilogue
+constexpr uint32_t kMergeBytes = (kEpiPerQuarter - 1) * 2 * kBM * 20;  // row states handed over at the end of a sweep
 constexpr uint32_t kStageBytesA = kBM * kBK * 2;  // 16 KB of H per stage
 constexpr uint32_t kScoreSmemMax = 227u * 1024u;  // the most dynamic shared memory a CTA may have
 constexpr uint32_t kSmemOverhead = 1024 /* ring alignment slack */ + 256 /* barriers */;

@@ -390,6 +390,29 @@ __device__ __forceinline__ float ex2(float x)
     return y;
 }
 
+// Two fp32 operations per instruction, each rounded as the scalar one: a * b + c and a + b.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    union { float2 f; uint64_t u; } x{a}, y{b}, z{c}, d;
+    asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(d.u) : "l"(x.u), "l"(y.u), "l"(z.u));
+    return d.f;
+}
+
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    union { float2 f; uint64_t u; } x{a}, y{b}, d;
+    asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(d.u) : "l"(x.u), "l"(y.u));
+    return d.f;
+}
+
+// max of three (a NaN operand is ignored, as by fmaxf).
+__device__ __forceinline__ float max3(float a, float b, float c)
+{
+    float d;
+    asm("max.ftz.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
 // log2(x) on the special-function unit (lg2.approx: max absolute error about 2^-22 near 1).
 __device__ __forceinline__ float lg2(float x)
 {

@@ -6,7 +6,7 @@
 // The logits never leave the chip: each CTA pair computes logit tiles of 256
 // rows x bn vocabulary columns with 2-SM tensor-core MMAs
 // (tcgen05.mma.cta_group::2, bf16 x bf16 -> fp32 in TMEM, M = 256 split
-// 128/128 over the two SMs, N = bn <= 256), and four epilogue warps per CTA
+// 128/128 over the two SMs, N = bn <= 256), and eight epilogue warps per CTA
 // fold each tile straight out of TMEM into a running per-row state (max, sum
 // of exp, argmax, target logit) that lives in registers across all of the
 // pair's vocabulary tiles of that row block.  One partial record per
@@ -33,7 +33,7 @@
 //     deferred until the epilogue has read that one too (the stages are
 //     released after those).
 //
-// Kernel structure (persistent, clusters of 2 CTAs = one SM pair, 192 threads each):
+// Kernel structure (persistent, clusters of 2 CTAs = one SM pair, 320 threads each):
 //   warp 0  TMA producer (both CTAs): per K slice, its 128 rows of H (of one
 //           or two row blocks) and its bn/2 of the (one or two) tiles' W rows
 //           into the ring; both CTAs' copies complete on the LEADER's stage
@@ -51,9 +51,18 @@
 //           full clock; d = 4096, V = 126464): N = 64 168 -> 156, N = 256
 //           179 -> 166, N = 2048 1092 -> 1070; d = 1024, V = 64000, N = 2048
 //           247 -> 201;
-//   warps 2-5 epilogue (both CTAs): one thread per row (TMEM lane); online
-//           softmax over a tile's columns, then release of the accumulator to
-//           the leader's MMA warp (8 arrivals per accumulator use).
+//   warps 2-9 epilogue (both CTAs): two warps per TMEM lane quarter, on the
+//           even and the odd 32-column chunks of every tile; one thread per row
+//           (TMEM lane) and warp.  Online softmax over its chunks, then release
+//           of the accumulator to the leader's MMA warp.  At the end of a sweep
+//           the second warp's row states are merged into the first one's.
+//           The epilogue is latency-bound in a single warp per scheduler (25-30
+//           cycles per column against 5 instructions), and a pass's MMAs wait
+//           for it.  One warp per quarter, then two with the packed fold of
+//           fold.cuh and accumulator 0 handed over before accumulator 1 is
+//           done (us per step, V = 64000, N = 2048): d = 256 107 -> 74, d = 1024
+//           200 -> 182; d = 4096, V = 126464 1195 -> 1173; three or four warps
+//           per quarter: 72 / 73, 182 / 183, no change.
 // Work split: see ScoreArgs in internal.h.
 //
 // Every mbarrier wait is bounded (kWaitLimitNs): on expiry the CTA raises an
@@ -78,38 +87,38 @@ namespace {
 
 constexpr uint16_t kBothCtas = 0x3;
 constexpr int kPrefetchSlices = 4;   // K slices of the first W tile prefetched into L2 before the grid wait
-constexpr int kTmemLoadsPerWait = 1;  // 32-column TMEM loads in flight per tcgen05.wait::ld in the epilogue (2 measured slower)
 
 struct alignas(8) Barriers {
     uint64_t full[kMaxStages];   // leader: both CTAs' copies of a stage landed
     uint64_t empty[kMaxStages];  // both: the stage's MMAs are done (multicast commit)
     uint64_t tmem_full[2];       // both: accumulator i holds a finished tile (multicast commit)
-    uint64_t tmem_empty[2];      // leader: all 8 epilogue warps of the pair have read accumulator i
+    uint64_t tmem_empty[2];      // leader: every epilogue warp of the pair has read accumulator i
     uint64_t mma_done;           // leader: every MMA issued has completed
     uint32_t tmem_base;
     int32_t abort;
 };
 static_assert(sizeof(Barriers) <= 256, "barrier block must fit its reserve");
 
-// Fold the nvalid first columns of one accumulator (this warp's 32 TMEM lanes from tbase), vocabulary
-// ids v0 ..; kTmemLoadsPerWait 32-column loads in flight per wait.
+// Fold this warp's share of the nvalid first columns of one accumulator (32 TMEM lanes from tbase), vocabulary ids
+// v0 ..: every kEpiPerQuarter-th 32-column chunk from chunk `sel` on.
 template <bool kEntropy>
-__device__ __forceinline__ void fold_tile(RowState &r, uint32_t tbase, int v0, int nvalid, int tgt)
+__device__ __forceinline__ void fold_tile(RowState &r, uint32_t tbase, int sel, int v0, int nvalid, int tgt)
 {
 #pragma unroll 1
-    for (int c = 0; c * 32 < nvalid; c += kTmemLoadsPerWait) {
-        float x[kTmemLoadsPerWait][32];
-#pragma unroll
-        for (int i = 0; i < kTmemLoadsPerWait; ++i)
-            if (i == 0 || (c + i) * 32 < nvalid)  // warp-uniform
-                ptx::tmem_ld_32x32b_x32(tbase + (uint32_t)((c + i) * 32), x[i]);
+    for (int c = sel * 32; c < nvalid; c += 32 * kEpiPerQuarter) {
+        float x[32];
+        ptx::tmem_ld_32x32b_x32(tbase + (uint32_t)c, x);
         ptx::tmem_ld_wait();
-#pragma unroll
-        for (int i = 0; i < kTmemLoadsPerWait; ++i)
-            if (i == 0 || (c + i) * 32 < nvalid)
-                fold32<kEntropy>(r, x[i], v0 + (c + i) * 32, nvalid - (c + i) * 32, tgt);
+        fold32<kEntropy>(r, x, v0 + c, nvalid - c, tgt);
     }
 }
+
+// One row's state as the other epilogue warps of its lane quarter hand it over.
+struct RowPart {
+    float m[kBM], s[kBM], tlog[kBM], u[kBM];
+    int32_t am[kBM];
+};
+static_assert(2 * (kEpiPerQuarter - 1) * sizeof(RowPart) == kMergeBytes, "merge scratch");
 
 // kTwo: passes (ScoreArgs::two == 1: row-pair and tile-pair sweeps), else single tiles.
 template <bool kEntropy, bool kTwo>
@@ -120,7 +129,11 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = ptx::smem_u32(smem_raw);
     const uint32_t ring = (raw + 1023u) & ~1023u;  // swizzle atoms need 1024-B alignment
-    Barriers *bars = reinterpret_cast<Barriers *>(smem_raw + (ring - raw) + (uint32_t)a.stages * a.stage_bytes);
+    const uint32_t ring_bytes = (uint32_t)a.stages * a.stage_bytes;
+    Barriers *bars = reinterpret_cast<Barriers *>(smem_raw + (ring - raw) + ring_bytes + (kTwo ? kMergeBytes : 0u));
+    // Scratch for merging a row's states at the end of a sweep.  Single tiles have one sweep per launch, at whose end
+    // the ring is free.
+    RowPart *const parts = reinterpret_cast<RowPart *>(smem_raw + (ring - raw) + (kTwo ? ring_bytes : 0u));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = ptx::cluster_ctarank();  // 0: leader (issues the MMAs), 1: peer
     const bool leader = rank == 0;
@@ -152,7 +165,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
         }
         for (int i = 0; i < 2; ++i) {
             ptx::mbar_init(tfull(i), 1);
-            ptx::mbar_init(tempty(i), 8);  // 4 epilogue warps in each CTA of the pair
+            ptx::mbar_init(tempty(i), 2 * kEpiWarps);  // the epilogue warps of both CTAs
         }
         ptx::mbar_init(mma_done, 1);
         bars->abort = 0;
@@ -198,8 +211,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
             a.status->finished = 0;  // the previous call's finish kernel has completed
         if (tl && threadIdx.x == 64)
             tl[3] = ptx::globaltimer_ns();
-        for (int i = blockIdx.x * 128 + (int)threadIdx.x - 64; i < a.n_tickets; i += gridDim.x * 128)
-            if (threadIdx.x >= 64)
+        if (threadIdx.x >= 64)
+            for (int i = blockIdx.x * (32 * kEpiWarps) + (int)threadIdx.x - 64; i < a.n_tickets;
+                 i += gridDim.x * (32 * kEpiWarps))
                 a.tickets[i] = 0;
     }
     if (!tmem_ok) {
@@ -309,6 +323,8 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
                             break;
                         }
                         issue(acc0, sA(stage), sB(stage, 0), kb);
+                        if (kb == a.n_kb - 1)  // accumulator 0 is done: its epilogue need not wait for accumulator 1
+                            ptx::mma_commit_pair_multicast(tfull(acc0), kBothCtas);
                         if (kb < defer) {
                             if (kb == defer - 1) {  // the second accumulator is needed now
                                 if (!wait_acc_free(1, (uint32_t)item)) {
@@ -335,7 +351,6 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
                     }
                     if (aborted)
                         break;
-                    ptx::mma_commit_pair_multicast(tfull(acc0), kBothCtas);
                     if (kTwo)  // the epilogue waits for both accumulators of every pass
                         ptx::mma_commit_pair_multicast(tfull(1), kBothCtas);
                     tiles += two ? 2 : 1;
@@ -351,8 +366,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
         }
         __syncwarp();
     } else {
-        // ------------------------------------------------------------ epilogue (warps 2..5, both CTAs)
-        const int q = warp & 3;  // this warp may only read TMEM lanes [32q, 32q + 32)
+        // ------------------------------------------------------------ epilogue (warps 2.., both CTAs)
+        const int q = warp & 3;           // this warp may only read TMEM lanes [32q, 32q + 32)
+        const int sel = (warp - 2) >> 2;  // which of the quarter's warps
         const uint32_t lanes = tmem + ((uint32_t)(q * 32) << 16);
         int item = 0;
         bool aborted = false;
@@ -370,8 +386,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
             if (lane == 0)
                 ptx::mbar_arrive_cluster(ptx::mapa(tempty(i), 0));
         };
+        auto epilogue_sync = [&] { asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory"); };
         const RowState r0{-INFINITY, 0.f, 0.f, 0.f, 0.f, -INFINITY, 0.f, 0.f, 0.f, 0.f, 0};
-        for (int mb = grp; mb < a.n_mb && !aborted; mb += mb_step) {
+        for (int mb = grp; mb < a.n_mb; mb += mb_step) {
             const int mb2 = mb + a.n_groups;
             const bool rows2 = kTwo && mb2 < a.n_mb;
             const int64_t in_block = (int)rank * kBM + q * 32 + lane;
@@ -380,14 +397,14 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
             const int32_t tgt = (row < a.N) ? row_target(a.ts, row, a.V) : -1;
             const int32_t tgt2 = (row2 < a.N) ? row_target(a.ts, row2, a.V) : -1;
             RowState r = r0, r2 = r0;  // r2: the partner block's row in a row-pair sweep
-            for (int vt = col; vt < a.n_vt; vt += rows2 ? a.G : vstep, ++item) {
+            for (int vt = col; vt < a.n_vt && !aborted; vt += rows2 ? a.G : vstep, ++item) {
                 const int acc0 = kTwo ? 0 : (item & 1);
                 const uint32_t uses0 = kTwo ? (uint32_t)item : (uint32_t)(item >> 1);
                 if (!take(acc0, uses0)) {
                     aborted = true;
                     break;
                 }
-                fold_tile<kEntropy>(r, lanes + (uint32_t)acc0 * kBN, vt * a.bn, min(a.bn, a.V - vt * a.bn), tgt);
+                fold_tile<kEntropy>(r, lanes + (uint32_t)acc0 * kBN, sel, vt * a.bn, min(a.bn, a.V - vt * a.bn), tgt);
                 release(acc0);
                 if (kTwo) {
                     if (!take(1, (uint32_t)item)) {
@@ -396,27 +413,56 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
                     }
                     const int vt1 = vt + a.G;
                     if (rows2)
-                        fold_tile<kEntropy>(r2, lanes + kBN, vt * a.bn, min(a.bn, a.V - vt * a.bn), tgt2);
+                        fold_tile<kEntropy>(r2, lanes + kBN, sel, vt * a.bn, min(a.bn, a.V - vt * a.bn), tgt2);
                     else if (vt1 < a.n_vt)
-                        fold_tile<kEntropy>(r, lanes + kBN, vt1 * a.bn, min(a.bn, a.V - vt1 * a.bn), tgt);
+                        fold_tile<kEntropy>(r, lanes + kBN, sel, vt1 * a.bn, min(a.bn, a.V - vt1 * a.bn), tgt);
                     release(1);
                 }
             }
-            if (aborted)
-                break;
+            // Merge the states of the quarter's warps into the first one's.  (Every warp of the CTA comes here as
+            // often, aborted or not; after an abort the records are not used.)
+            if (sel > 0)
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {  // the previous sweep's records, then this sweep's become pending
-                if (pend_idx[i] >= 0) {
-                    a.part[pend_idx[i]] = pend[i];
+                for (int i = 0; i < (kTwo ? 2 : 1); ++i) {
+                    RowPart &p = parts[(sel - 1) * 2 + i];
+                    const RowState &x = i ? r2 : r;
+                    const int k = q * 32 + lane;
+                    p.m[k] = x.m;
+                    p.s[k] = (x.s0 + x.s1) + (x.s2 + x.s3);
+                    p.tlog[k] = x.tlog;
+                    p.am[k] = x.am;
                     if (kEntropy)
-                        a.part_u[pend_idx[i]] = pend_u[i];
+                        p.u[k] = (x.u0 + x.u1) + (x.u2 + x.u3);
                 }
-                const RowState &x = i ? r2 : r;
-                pend[i] = make_float4(x.m, (x.s0 + x.s1) + (x.s2 + x.s3), __int_as_float(x.am), x.tlog);
-                pend_u[i] = (x.u0 + x.u1) + (x.u2 + x.u3);
-                const int64_t rr = i ? row2 : row;
-                pend_idx[i] = rr < a.N ? rr * a.G + col : -1;
-            }
+            epilogue_sync();
+            if (sel == 0)
+#pragma unroll
+                for (int i = 0; i < (kTwo ? 2 : 1); ++i) {
+                    if (pend_idx[i] >= 0) {  // the previous sweep's records, then this sweep's become pending
+                        a.part[pend_idx[i]] = pend[i];
+                        if (kEntropy)
+                            a.part_u[pend_idx[i]] = pend_u[i];
+                    }
+                    const RowState &x = i ? r2 : r;
+                    float m = x.m, s = (x.s0 + x.s1) + (x.s2 + x.s3), t = x.tlog, u = (x.u0 + x.u1) + (x.u2 + x.u3);
+                    int32_t am = x.am;
+#pragma unroll
+                    for (int j = 0; j < kEpiPerQuarter - 1; ++j) {
+                        const RowPart &p = parts[j * 2 + i];
+                        const int k = q * 32 + lane;
+                        if (kEntropy)
+                            combine_u(m, s, u, am, p.m[k], p.s[k], p.u[k], p.am[k]);
+                        else
+                            combine(m, s, am, p.m[k], p.s[k], p.am[k]);
+                        t = fmaxf(t, p.tlog[k]);
+                    }
+                    pend[i] = make_float4(m, s, __int_as_float(am), t);
+                    pend_u[i] = u;
+                    const int64_t rr = i ? row2 : row;
+                    pend_idx[i] = rr < a.N ? rr * a.G + col : -1;
+                }
+            if (kTwo)
+                epilogue_sync();  // before the next sweep's states overwrite the scratch
         }
         if (tl && !leader && warp == 2 && lane == 0)
             tl[4] = ptx::globaltimer_ns();
@@ -497,9 +543,10 @@ ScoreSchedule score_schedule(int32_t n_mb, int64_t V, int max_units, int32_t rec
     // A pass stage has a third slot: the second tile's W, or in a row-pair sweep (a group with more than
     // one row block) the partner block's H.
     const uint32_t wb = stage_bytes_w(best.bn);
+    const uint32_t capacity = kRingCapacity - (two ? kMergeBytes : 0u);
     const bool row_pairs = two && n_mb > best.n_groups;
     best.stage_bytes = kStageBytesA + wb + (two ? (row_pairs && wb < kStageBytesA ? kStageBytesA : wb) : 0u);
-    const uint32_t fit = kRingCapacity / best.stage_bytes;
+    const uint32_t fit = capacity / best.stage_bytes;
     best.stages = (int32_t)(fit < (uint32_t)kMaxStages ? fit : (uint32_t)kMaxStages);
     return best;
 }
@@ -566,13 +613,15 @@ cudaError_t launch_score(const CUtensorMap &tmH, const CUtensorMap &tmW, const S
     // The ring must hold what the producer stages: a pass's third slot takes an H box (16 KB) in a row-pair
     // sweep, which the launch has when a group owns more than one row block.
     const uint32_t wb = stage_bytes_w(a.bn);
+    const uint32_t merge = a.two ? kMergeBytes : 0u;
     const uint32_t third = a.two ? (a.n_mb > a.n_groups && wb < kStageBytesA ? kStageBytesA : wb) : 0u;
     if (a.stages < 2 || a.stages > kMaxStages || a.stage_bytes < kStageBytesA + wb + third ||
-        a.stage_bytes % 1024u != 0 || (uint64_t)a.stages * a.stage_bytes > kRingCapacity)
+        a.stage_bytes % 1024u != 0 || (uint64_t)a.stages * a.stage_bytes > kRingCapacity - merge ||
+        (uint64_t)a.stages * a.stage_bytes < kMergeBytes)
         return cudaErrorInvalidValue;
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = score_launch_config((unsigned)(2 * a.n_groups * a.G), kScoreThreads,
-                                                 kSmemOverhead + (uint32_t)a.stages * a.stage_bytes, stream, attr);
+                                                 kSmemOverhead + merge + (uint32_t)a.stages * a.stage_bytes, stream, attr);
     if (entropy)
         return a.two ? cudaLaunchKernelEx(&cfg, score_kernel<true, true>, tmH, tmW, a)
                      : cudaLaunchKernelEx(&cfg, score_kernel<true, false>, tmH, tmW, a);

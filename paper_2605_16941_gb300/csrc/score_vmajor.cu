@@ -34,8 +34,8 @@ namespace {
 
 constexpr uint16_t kBothCtas = 0x3;
 constexpr int kPrefetchSlices = 4;  // K slices of the first W tile prefetched into L2 before the grid wait
-constexpr int kEpiWarps = 8;
-constexpr int kVmThreads = 64 + 32 * kEpiWarps;
+constexpr int kVmEpiWarps = 8;
+constexpr int kVmThreads = 64 + 32 * kVmEpiWarps;
 constexpr int kMaxChunks = 4;  // 32-column chunks of one accumulator (256 columns) per epilogue warp
 // The split and the choice between the two score kernels: ns per 64-wide K slice of a tile on the busiest pair, fitted
 // to steps in power-capped steady state (d = 4096, V = 126464; N from 128 to 2048, 1 to 8 groups; within 5 %):
@@ -53,7 +53,7 @@ constexpr int kVmMaxGroups = 8;
 constexpr int kVmEvenTileRows = 192;  // rows per group up to which the W stream, not the MMAs, sets the time: tiles are
                                       // then narrowed to split the vocabulary evenly over the pairs (V = 126464 on 76
                                       // pairs: 240; N = 300, MMA-bound: 242 us with 240, 236 with 256)
-constexpr uint32_t kTransBytes = kEpiWarps * 32 * 32 * 4;
+constexpr uint32_t kTransBytes = kVmEpiWarps * 32 * 32 * 4;
 
 struct alignas(8) VmBarriers {
     uint64_t full[kVmMaxStages];       // leader: both CTAs' copies of a stage landed
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kVmThreads, 1)
         }
         for (int i = 0; i < kVmMaxSlots; ++i) {
             ptx::mbar_init(tfull(i), 1);
-            ptx::mbar_init(tempty(i), 2 * kEpiWarps);  // the epilogue warps of both CTAs
+            ptx::mbar_init(tempty(i), 2 * kVmEpiWarps);  // the epilogue warps of both CTAs
         }
         ptx::mbar_init(mma_done, 1);
         bars->abort = 0;
@@ -164,8 +164,8 @@ __global__ void __launch_bounds__(kVmThreads, 1)
         if (tl && threadIdx.x == 64)
             tl[3] = ptx::globaltimer_ns();
         if (threadIdx.x >= 64)
-            for (int i = blockIdx.x * (32 * kEpiWarps) + (int)threadIdx.x - 64; i < a.n_tickets;
-                 i += gridDim.x * (32 * kEpiWarps))
+            for (int i = blockIdx.x * (32 * kVmEpiWarps) + (int)threadIdx.x - 64; i < a.n_tickets;
+                 i += gridDim.x * (32 * kVmEpiWarps))
                 a.tickets[i] = 0;
     }
     if (!tmem_ok) {
@@ -262,6 +262,8 @@ __global__ void __launch_bounds__(kVmThreads, 1)
                         break;
                     }
                     issue(acc0, stage, 0, kb);
+                    if (kb == a.n_kb - 1)  // accumulator 0 is done: its epilogue need not wait for accumulator 1
+                        ptx::mma_commit_pair_multicast(tfull(acc0), kBothCtas);
                     if (second) {
                         if (halves == 2)
                             issue(acc1, stage, 1, kb);
@@ -295,7 +297,6 @@ __global__ void __launch_bounds__(kVmThreads, 1)
                 }
                 if (aborted)
                     break;
-                ptx::mma_commit_pair_multicast(tfull(acc0), kBothCtas);
                 if (halves == 2)
                     ptx::mma_commit_pair_multicast(tfull(acc1), kBothCtas);
                 ++tiles;
@@ -402,7 +403,7 @@ __global__ void __launch_bounds__(kVmThreads, 1)
             if (kEntropy)
                 rec_u[q * kVmMaxRows + c] = st[k].u;
         }
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kVmEpiWarps) : "memory");
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const int c = (int)threadIdx.x - 64, row = row_of(i, c);  // column c of accumulator i
