@@ -12,11 +12,11 @@
 // CTA then adds its merged rows to its sequences' tickets; the CTA that
 // completes a sequence's 2*L_b rows applies Eq. 4 to that sequence, so merge
 // and update need one launch.  Tickets are cleared by the score kernel of the
-// same step.  The kernel is launched programmatically: its launch overlaps the
-// score kernel and it waits (griddepcontrol.wait) for the score kernel's
+// same step.  The kernel is launched programmatically: its CTAs start beside the
+// score kernel's and wait (griddepcontrol.wait) for the score kernel's
 // results before touching them; it lets the next call's kernels launch at once
-// (they only read H and W before their own griddepcontrol.wait).  The last of
-// its CTAs publishes the call's status (see StatusWords).
+// (they only prefetch W before their own griddepcontrol.wait).  The last of
+// its CTAs to merge its rows publishes the call's status (see StatusWords).
 //
 // draft_verify_kernel: Eq. 4 alone from caller-supplied statistics
 // (wino_draft_verify), one CTA per sequence.
@@ -43,13 +43,18 @@ namespace {
 
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr int kFinishRows = 8;  // rows (warps) per finish CTA; also the CTA size of the Eq. 4 kernels
+constexpr int kRecInFlight = 5;  // records each lane loads at once (160 per row: two per pair of a 76-pair launch fit)
 
 // Block-wide reduction scratch for eq4_block.
 struct Eq4Smem {
     int32_t i0[kFinishRows], i1[kFinishRows], i2[kFinishRows];
     float f0[kFinishRows];
-    float conf[kMaxBlkLen];  // fixed-M drafting: pmax of each masked position, -inf elsewhere
 };
+
+// Dynamic shared memory of a launch with fixed-M drafting: pmax of each masked position, -inf elsewhere.  (Static, it
+// would keep the CTA from fitting beside a score CTA, see kScoreSmemMax.)
+extern __shared__ float s_conf[];
+inline uint32_t conf_bytes(const wino_params &p) { return p.draft_m > 0 ? (uint32_t)p.blk_len * 4u : 0u; }
 
 // Eq. 4 on sequence s by the whole CTA (kFinishRows warps; thread t owns positions t, t + 256, ...),
 // reading the statistics of the a-th sequence of the scored rows (a = s unless an active-sequence list
@@ -155,7 +160,7 @@ __device__ void eq4_block(int a, int s, int32_t *tokens, const int32_t *argmax, 
         for (int i = 0; i < kPer; ++i) {
             const int l = tid + i * kT;
             if (l < L)
-                sm.conf[l] = (yv[i] == mask) ? pm[i] : -INFINITY;
+                s_conf[l] = (yv[i] == mask) ? pm[i] : -INFINITY;
         }
         __syncthreads();
 #pragma unroll
@@ -164,7 +169,7 @@ __device__ void eq4_block(int a, int s, int32_t *tokens, const int32_t *argmax, 
             if (l < L && yv[i] == mask) {
                 int before = 0;
                 for (int j = 0; j < L && before < p.draft_m; ++j) {
-                    const float c = sm.conf[j];
+                    const float c = s_conf[j];
                     before += (c > pm[i]) || (c == pm[i] && j < l);
                 }
                 top[i] = before < p.draft_m;
@@ -223,15 +228,25 @@ __device__ void eq4_block(int a, int s, int32_t *tokens, const int32_t *argmax, 
     __syncthreads();  // the scratch may be reused for the next sequence
 }
 
-// Eq. 4: the CTA that merges the last rows of a sequence updates that sequence.
-__device__ void eq4_tail(const FinishArgs &a, int64_t row0, int32_t status, int32_t *s_done, int32_t &s_ndone,
-                         Eq4Smem &sm)
+// The status that invalidates this call's scores (WINO_ERR_ARG is the finish kernel's own, see bad_entry).
+__device__ __forceinline__ int32_t score_status(const StatusWords *w)
 {
-    __syncthreads();
+    const int32_t s = *reinterpret_cast<const volatile int32_t *>(&w->current);
+    return s == WINO_ERR_ARG ? (int32_t)WINO_OK : s;
+}
+
+// Whether the caller's active-sequence list names no sequence of the batch for the a-th scored sequence.
+__device__ __forceinline__ bool bad_entry(const wino_params &p, int64_t a)
+{
+    return p.active_seq && (p.active_seq[a] < 0 || p.active_seq[a] >= p.n_seq);
+}
+
+// Eq. 4: the CTA that merges the last rows of a sequence updates that sequence.
+__device__ void eq4_tail(const FinishArgs &a, int64_t row0, int64_t per_seq, int32_t status, int32_t *s_done,
+                         int32_t &s_ndone, Eq4Smem &sm)
+{
     if (threadIdx.x == 0) {
         int32_t nd = 0;
-        const int64_t per_seq =
-            ((a.p.options & (WINO_OPT_NO_SHADOW | WINO_OPT_COMPACT)) ? 1 : 2) * (int64_t)a.p.blk_len;
         const int64_t rend = min(row0 + kFinishRows, (int64_t)a.N);
         for (int64_t r = row0; r < rend;) {
             const int64_t sq = r / per_seq;
@@ -247,105 +262,90 @@ __device__ void eq4_tail(const FinishArgs &a, int64_t row0, int32_t status, int3
     __syncthreads();
     const int nd = s_ndone;
     for (int i = 0; i < nd; ++i) {
+        if (bad_entry(a.p, s_done[i]))
+            continue;  // no update (the status says so)
         const int sq = a.p.active_seq ? a.p.active_seq[s_done[i]] : s_done[i];
-        if (sq < 0 || sq >= a.p.n_seq) {  // a bad entry of the caller's list: no update, an error status
-            if (threadIdx.x == 0)
-                atomicExch(&a.status->current, (int32_t)WINO_ERR_ARG);
-            continue;
-        }
         eq4_block(s_done[i], sq, a.tokens, a.argmax, a.pmax, a.ptarget, a.p, a.counts, a.flags, status, sm);
     }
 }
 
-__global__ void __launch_bounds__(kFinishRows * 32) finish_kernel(const FinishArgs a)
+// What bounds it is latency: a chain of dependent round trips to L2 (records; tickets; statistics) after the score
+// kernel's last CTA.  Its CTAs are small enough in registers and shared memory to be resident beside the score CTAs
+// and wait there, the records are loaded without waiting for the status word, and the count of finished CTAs runs
+// beside the tickets and Eq. 4.  With 64 registers a thread and 4.3 KB of shared memory it started only when score CTAs
+// left their SMs.  us per step in a CUDA graph, before -> after: d = 64, V = 1000, N = 64 9.5 -> 8.5; d = 512,
+// V = 32000, N = 128 14.3 -> 13.3; d = 1024, V = 64000, N = 256 30.0 -> 29.2; nothing measurable from 150 us up.
+__global__ void __launch_bounds__(kFinishRows * 32, 5) finish_kernel(const FinishArgs a)
 {
     ptx::grid_dep_launch_dependents();  // the next call may start streaming its H and W
-    ptx::grid_dep_wait();
     __shared__ int32_t s_done[kFinishRows];
     __shared__ int32_t s_ndone;
     __shared__ Eq4Smem sm;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t row0 = (int64_t)blockIdx.x * kFinishRows;
     const int64_t row = row0 + warp;
-    const int32_t status = *reinterpret_cast<volatile int32_t *>(&a.status->current);
+    const int64_t per_seq =
+        ((a.p.options & (WINO_OPT_NO_SHADOW | WINO_OPT_COMPACT)) ? 1 : 2) * (int64_t)a.p.blk_len;  // rows
+    ptx::grid_dep_wait();
+    const int32_t status = score_status(a.status);
 
     if (row < a.N) {
-        if (status != WINO_OK) {
-            if (lane == 0) {
-                a.argmax[row] = -1;
-                a.pmax[row] = __int_as_float(0x7fc00000);
-                a.ptarget[row] = __int_as_float(0x7fc00000);
-                if (a.entropy)
-                    a.entropy[row] = __int_as_float(0x7fc00000);
-            }
-        } else {
-            const float4 *pr = a.part + row * a.G;
-            // every record of the row (G <= 8 * 32) and the target's record are loaded at once
-            constexpr int kRec = kMaxRecordsPerRow / 32;
-            float4 r[kRec];
+        // Every record of the row (the workspace holds them whatever the status); the record of the pair whose tiles
+        // hold the row's target carries its logit, the others -inf.
+        const float4 *pr = a.part + row * a.G;
+        float m = -INFINITY, s = 0.f, tl = -INFINITY, u = 0.f;
+        int32_t idx = INT32_MAX;
+        for (int j0 = 0; j0 < a.G; j0 += 32 * kRecInFlight) {
+            float4 r[kRecInFlight];
 #pragma unroll
-            for (int i = 0; i < kRec; ++i) {
-                const int j = lane + 32 * i;
+            for (int i = 0; i < kRecInFlight; ++i) {
+                const int j = j0 + lane + 32 * i;
                 r[i] = (j < a.G) ? __ldcg(pr + j) : make_float4(-INFINITY, 0.f, __int_as_float(INT32_MAX), -INFINITY);
             }
-            // The record of the pair whose tiles hold the row's target carries its logit; the others -inf.
-            float m = -INFINITY, s = 0.f, tl = -INFINITY, u = 0.f;
-            int32_t idx = INT32_MAX;
-            if (!a.entropy) {
 #pragma unroll
-                for (int i = 0; i < kRec; ++i) {
+            for (int i = 0; i < kRecInFlight; ++i) {
+                const int j = j0 + lane + 32 * i;
+                if (!a.entropy)
                     combine(m, s, idx, r[i].x, r[i].y, __float_as_int(r[i].z));
-                    tl = fmaxf(tl, r[i].w);
-                }
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) {
-                    const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-                    const float s2 = __shfl_xor_sync(0xffffffffu, s, off);
-                    const int32_t i2 = __shfl_xor_sync(0xffffffffu, idx, off);
-                    tl = fmaxf(tl, __shfl_xor_sync(0xffffffffu, tl, off));
-                    combine(m, s, idx, m2, s2, i2);
-                }
-            } else {
-                const float *pu = a.part_u + row * a.G;
-#pragma unroll
-                for (int i = 0; i < kRec; ++i) {
-                    const int j = lane + 32 * i;
-                    combine_u(m, s, u, idx, r[i].x, r[i].y, (j < a.G) ? __ldcg(pu + j) : 0.f,
-                              __float_as_int(r[i].z));
-                    tl = fmaxf(tl, r[i].w);
-                }
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) {
-                    const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-                    const float s2 = __shfl_xor_sync(0xffffffffu, s, off);
-                    const float u2 = __shfl_xor_sync(0xffffffffu, u, off);
-                    const int32_t i2 = __shfl_xor_sync(0xffffffffu, idx, off);
-                    tl = fmaxf(tl, __shfl_xor_sync(0xffffffffu, tl, off));
-                    combine_u(m, s, u, idx, m2, s2, u2, i2);
-                }
-            }
-            if (lane == 0) {
-                a.argmax[row] = idx;
-                a.pmax[row] = 1.0f / s;
-                a.ptarget[row] = (tl > -INFINITY) ? ptx::ex2((tl - m) * kLog2e) / s : 0.0f;
-                if (a.entropy)  // H = ln Z - (u ln 2) / Z, with u in log2 units
-                    a.entropy[row] = (ptx::lg2(s) - u / s) * kLn2;
-                __threadfence();  // publish this row before the CTA signals its ticket
+                else
+                    combine_u(m, s, u, idx, r[i].x, r[i].y,
+                              (j < a.G) ? __ldcg(a.part_u + row * a.G + j) : 0.f, __float_as_int(r[i].z));
+                tl = fmaxf(tl, r[i].w);
             }
         }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
+            const float s2 = __shfl_xor_sync(0xffffffffu, s, off);
+            const int32_t i2 = __shfl_xor_sync(0xffffffffu, idx, off);
+            tl = fmaxf(tl, __shfl_xor_sync(0xffffffffu, tl, off));
+            if (!a.entropy)
+                combine(m, s, idx, m2, s2, i2);
+            else
+                combine_u(m, s, u, idx, m2, s2, __shfl_xor_sync(0xffffffffu, u, off), i2);
+        }
+        if (lane == 0) {
+            const bool ok = status == WINO_OK;
+            const float nan = __int_as_float(0x7fc00000);
+            a.argmax[row] = ok ? idx : -1;
+            a.pmax[row] = ok ? 1.0f / s : nan;
+            a.ptarget[row] = !ok ? nan : ((tl > -INFINITY) ? ptx::ex2((tl - m) * kLog2e) / s : 0.0f);
+            if (a.entropy)  // H = ln Z - (u ln 2) / Z, with u in log2 units
+                a.entropy[row] = ok ? (ptx::lg2(s) - u / s) * kLn2 : nan;
+            if (a.tokens && bad_entry(a.p, row / per_seq))  // reported unless the scores already failed
+                atomicCAS(&a.status->current, (int32_t)WINO_OK, (int32_t)WINO_ERR_ARG);
+            __threadfence();  // publish this row and the status before the CTA signals its ticket and its end
+        }
+    }
+    __syncthreads();
+    // The last CTA to come here publishes the call's status and clears the word for the next call: every CTA has read
+    // the word, and recorded its own errors, before.
+    if (threadIdx.x == 32 && atomicAdd(&a.status->finished, 1u) == gridDim.x - 1) {
+        __threadfence();
+        a.status->last = atomicExch(&a.status->current, (int32_t)WINO_OK);
     }
     if (a.tokens)
-        eq4_tail(a, row0, status, s_done, s_ndone, sm);
-
-    // The last CTA done with this call publishes its status and clears the word for the next call.
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        if (atomicAdd(&a.status->finished, 1u) == gridDim.x - 1) {
-            __threadfence();
-            a.status->last = atomicExch(&a.status->current, (int32_t)WINO_OK);
-        }
-    }
+        eq4_tail(a, row0, per_seq, status, s_done, s_ndone, sm);
 }
 
 // Eq. 4 alone, one CTA per sequence.
@@ -451,7 +451,7 @@ cudaError_t launch_finish(const FinishArgs &a, cudaStream_t stream)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((a.N + kFinishRows - 1) / kFinishRows));
     cfg.blockDim = dim3(kFinishRows * 32);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = a.tokens ? conf_bytes(a.p) : 0;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -464,7 +464,7 @@ cudaError_t launch_finish(const FinishArgs &a, cudaStream_t stream)
 cudaError_t launch_draft_verify(int32_t *tokens, const int32_t *argmax, const float *pmax, const float *ptarget,
                                 const wino_params &p, int32_t *counts, int8_t *flags, cudaStream_t stream)
 {
-    draft_verify_kernel<<<p.n_seq, kFinishRows * 32, 0, stream>>>(tokens, argmax, pmax, ptarget, p, counts, flags);
+    draft_verify_kernel<<<p.n_seq, kFinishRows * 32, conf_bytes(p), stream>>>(tokens, argmax, pmax, ptarget, p, counts, flags);
     return cudaGetLastError();
 }
 

@@ -37,9 +37,12 @@ constexpr int kEpiWarps = 4 * kEpiPerQuarter;
 constexpr int kScoreThreads = 64 + 32 * kEpiWarps;  // warp 0 TMA, warp 1 TMEM + MMA, then the epilogue
 constexpr uint32_t kMergeBytes = (kEpiPerQuarter - 1) * 2 * kBM * 20;  // row states handed over at the end of a sweep
 constexpr uint32_t kStageBytesA = kBM * kBK * 2;  // 16 KB of H per stage
-constexpr uint32_t kScoreSmemMax = 227u * 1024u;  // the most dynamic shared memory a CTA may have
+constexpr uint32_t kSmemLimit = 227u * 1024u;  // the most dynamic shared memory a CTA may have
+// What a score CTA takes at most (a few pass-mode widths excepted), so that a finish CTA (1 KB reserved + 256 B static) fits beside it in an SM's 228 KB.
+constexpr uint32_t kScoreSmemMax = kSmemLimit - 1280u;
 constexpr uint32_t kSmemOverhead = 1024 /* ring alignment slack */ + 256 /* barriers */;
 constexpr uint32_t kRingCapacity = kScoreSmemMax - kSmemOverhead;
+constexpr uint32_t kPassRingCapacity = kSmemLimit - kSmemOverhead - kMergeBytes;  // a stage more (bn = 224) is worth more
 constexpr uint32_t kTmemCols = 2 * kBN;  // two 256-column fp32 accumulators: all 512 TMEM columns
 
 // W bytes one CTA stages per K slice of a tile of width bn (bn/2 rows of 128 B; a multiple of 1 KB).

@@ -543,7 +543,7 @@ ScoreSchedule score_schedule(int32_t n_mb, int64_t V, int max_units, int32_t rec
     // A pass stage has a third slot: the second tile's W, or in a row-pair sweep (a group with more than
     // one row block) the partner block's H.
     const uint32_t wb = stage_bytes_w(best.bn);
-    const uint32_t capacity = kRingCapacity - (two ? kMergeBytes : 0u);
+    const uint32_t capacity = two ? kPassRingCapacity : kRingCapacity;
     const bool row_pairs = two && n_mb > best.n_groups;
     best.stage_bytes = kStageBytesA + wb + (two ? (row_pairs && wb < kStageBytesA ? kStageBytesA : wb) : 0u);
     const uint32_t fit = capacity / best.stage_bytes;
@@ -585,12 +585,12 @@ int configure_device()
     if (!done[dev]) {
         for (auto *k : {score_kernel<false, false>, score_kernel<false, true>, score_kernel<true, false>,
                         score_kernel<true, true>})
-            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScoreSmemMax) !=
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) !=
                 cudaSuccess)
                 return -1;
         cudaLaunchAttribute attr[2];
         // Any launch's shared memory exceeds half an SM's, so one CTA per SM whatever the ring size.
-        cudaLaunchConfig_t cfg = score_launch_config(2, kScoreThreads, kScoreSmemMax, nullptr, attr);
+        cudaLaunchConfig_t cfg = score_launch_config(2, kScoreThreads, kSmemLimit, nullptr, attr);
         cfg.numAttrs = 1;  // the cluster shape is what matters for the occupancy query
         int clusters = 0;
         if (cudaOccupancyMaxActiveClusters(&clusters, score_kernel<false, true>, &cfg) != cudaSuccess || clusters < 1)
@@ -616,7 +616,7 @@ cudaError_t launch_score(const CUtensorMap &tmH, const CUtensorMap &tmW, const S
     const uint32_t merge = a.two ? kMergeBytes : 0u;
     const uint32_t third = a.two ? (a.n_mb > a.n_groups && wb < kStageBytesA ? kStageBytesA : wb) : 0u;
     if (a.stages < 2 || a.stages > kMaxStages || a.stage_bytes < kStageBytesA + wb + third ||
-        a.stage_bytes % 1024u != 0 || (uint64_t)a.stages * a.stage_bytes > kRingCapacity - merge ||
+        a.stage_bytes % 1024u != 0 || (uint64_t)a.stages * a.stage_bytes > (a.two ? kPassRingCapacity : kRingCapacity) ||
         (uint64_t)a.stages * a.stage_bytes < kMergeBytes)
         return cudaErrorInvalidValue;
     cudaLaunchAttribute attr[2];
