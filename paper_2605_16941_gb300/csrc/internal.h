@@ -210,7 +210,7 @@ cudaError_t launch_gather_compact(const uint16_t *H, uint16_t *Hc, const int32_t
                                   int64_t d, cudaStream_t stream);
 
 // Wp[k][v][c] = W[v][64k + c] (wino_lm_head_panels); d a multiple of 64, (d/64) * V <= 2^30.
-cudaError_t launch_panels(const uint16_t *W, uint16_t *Wp, int64_t d, int64_t V, int sm_count, cudaStream_t stream);
+cudaError_t launch_panels(const uint16_t *W, uint16_t *Wp, int64_t d, int64_t V, cudaStream_t stream);
 
 cudaError_t launch_draft_verify(int32_t *tokens, const int32_t *argmax, const float *pmax, const float *ptarget,
                                 const wino_params &p, int32_t *counts, int8_t *flags, cudaStream_t stream);

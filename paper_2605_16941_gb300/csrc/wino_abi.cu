@@ -488,7 +488,7 @@ int wino_lm_head_panels(const uint16_t *W, int64_t d, int64_t V, uint16_t *Wp, v
     int rc = device_info(&info);
     if (rc != WINO_OK)
         return rc;
-    if (launch_panels(W, Wp, d, V, info.sm_count, static_cast<cudaStream_t>(stream)) != cudaSuccess)
+    if (launch_panels(W, Wp, d, V, static_cast<cudaStream_t>(stream)) != cudaSuccess)
         return WINO_ERR_CUDA;
     return WINO_OK;
 }

@@ -28,6 +28,22 @@ def test_panel_copy_is_the_permutation(V, d):
     assert torch.equal(Wp.view(torch.int16), ref.view(torch.int16))
 
 
+@pytest.mark.parametrize("d", [448, 512, 576, 1088])
+@pytest.mark.parametrize("V", [2, 31, 32, 257])
+def test_panel_copy_tile_edges(V, d):
+    """Rows and panels that fill, miss or run past a tile of the copy (32 rows x 8 panels, 256 x 1 below 8 panels), with
+    guard zones around the destination."""
+    import paper_2605_16941_gb300 as wino
+    from gpu_helpers import dev
+    W = dev(ws.random_bf16(V, d, 1.0 / d, seed=V + d))
+    buf = torch.full((64 + V * d + 64,), -7, dtype=torch.int16, device="cuda")
+    wino.wino_lm_head_panels(W, Wp=buf[64:64 + V * d].view(d // 64, V, 64))
+    torch.cuda.synchronize()
+    ref = W.view(V, d // 64, 64).permute(1, 0, 2).reshape(-1)
+    assert torch.equal(buf[64:64 + V * d], ref.view(torch.int16))
+    assert torch.all(buf[:64] == -7) and torch.all(buf[64 + V * d:] == -7)
+
+
 def _step_pair(w, H, W, Wp, st, **opts):
     """One step from the same state with row-major W and with the panel copy: (tokens, counts, flags, ws)."""
     import paper_2605_16941_gb300 as wino
