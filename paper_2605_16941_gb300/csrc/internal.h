@@ -164,7 +164,6 @@ struct ScoreSchedule {
     int32_t bn, n_vt, n_groups, G;
     int32_t two, stages;
     uint32_t stage_bytes;
-    int64_t cost;  // accumulator columns on the busiest pair, overheads included
 };
 ScoreSchedule score_schedule(int32_t n_mb, int64_t V, int max_units, int32_t records_cap);
 
@@ -174,7 +173,7 @@ struct VmSchedule {
     int32_t bn, n_vt, n_groups, G;
     int32_t hw[2], slots, stages;
     uint32_t stage_bytes;
-    int64_t cost;
+    int64_t cost;  // estimated ns
 };
 bool score_vmajor_schedule(int64_t N, int64_t d, int64_t V, int max_units, int32_t records_cap,
                            const ScoreSchedule &rows, VmSchedule *out);

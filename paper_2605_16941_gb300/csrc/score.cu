@@ -515,7 +515,7 @@ ScoreSchedule score_schedule(int32_t n_mb, int64_t V, int max_units, int32_t rec
     constexpr int64_t kTileOverheadCols = 16;  // single tiles: H re-staged per tile, in columns
     constexpr int64_t kPassOverheadCols = 32;  // passes: the epilogue the next pass partly waits for
     const int32_t two = n_mb >= kPassMinRowBlocks ? 1 : 0;
-    ScoreSchedule best{kBN, (int32_t)((V + kBN - 1) / kBN), 1, 1, two, 2, 0, 0};
+    ScoreSchedule best{kBN, (int32_t)((V + kBN - 1) / kBN), 1, 1, two, 2, 0};
     int64_t best_cost = -1;
     const int32_t top = n_mb < max_units ? n_mb : max_units;
     for (int32_t bn = kBN; bn >= kMinBN; bn -= 16) {
@@ -539,7 +539,6 @@ ScoreSchedule score_schedule(int32_t n_mb, int64_t V, int max_units, int32_t rec
             }
         }
     }
-    best.cost = best_cost;
     // A pass stage has a third slot: the second tile's W, or in a row-pair sweep (a group with more than
     // one row block) the partner block's H.
     const uint32_t wb = stage_bytes_w(best.bn);

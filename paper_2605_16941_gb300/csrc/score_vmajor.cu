@@ -37,18 +37,23 @@ constexpr int kPrefetchSlices = 4;  // K slices of the first W tile prefetched i
 constexpr int kVmEpiWarps = 8;
 constexpr int kVmThreads = 64 + 32 * kVmEpiWarps;
 constexpr int kMaxChunks = 4;  // 32-column chunks of one accumulator (256 columns) per epilogue warp
-// The split and the choice between the two score kernels: ns per 64-wide K slice of a tile on the busiest pair, fitted
-// to steps in power-capped steady state (d = 4096, V = 126464; N from 128 to 2048, 1 to 8 groups; within 5 %):
-// 130 + hw with one accumulator per tile, 75 + 1.4 (hw[0] + hw[1]) with two, and for score.cu a constant per tile of
-// 256 rows, fewer for a single block of 240-wide tiles.  us per step, score.cu -> here (groups): N = 32 157 -> 152 (1),
-// 128 168 -> 154 (1), 208 175 -> 171 (1), 256 183 -> 190 (stays with score.cu), 288 308 -> 220 (1), 320 316 -> 243 (1),
+// The split and the choice between the two score kernels: ns on the busiest pair, fitted to steps in steady state
+// (d = 4096, V = 126464, N from 128 to 2048, 1 to 8 groups; d = 256 to 1536 with V from 20000 to 64000; within 5 % of
+// most).  Per tile: n_kb K slices of 130 + hw with one accumulator, or the epilogue (15 ns a column) if that is longer,
+// as the accumulators alternate; 60 + 1.4 (hw[0] + hw[1]) with two, and part of their epilogue (4 ns a column).  Then
+// the last tile's epilogue.  score.cu: 380 per K slice of a 256-row tile, and 700 for its epilogue.
+// us per step, score.cu -> here (groups), d = 4096, V = 126464: N = 288 308 -> 220 (1), 320 316 -> 243 (1),
 // 384 326 -> 287 (1, 2), 448 333 -> 312 (2), 512 344 -> 346 (2), 576 494 -> 390 (2), 640 502 -> 421 (2),
-// 768 523 -> 482 (3), 896 616 -> 578 (4), 1024 632 -> 620 (4), 1280 870 -> 771 (5), 1536 953 -> 927 (6),
-// 1664 1171 -> 1036 (4), 2048 1204 -> 1213 (stays).
-constexpr int64_t kRowTileCost = 389;
-constexpr int64_t kRowTileCostOneBlock = 350;
-constexpr int kVmMinSlices = 24;            // K slices per tile that hide the transposing epilogue ...
-constexpr int kVmShortRows = 64;            // ... unless the rows are this few (d = 256, V = 64000, N = 64: 20.6 -> 16.7)
+// 768 523 -> 482 (3), 896 616 -> 578 (4), 1024 632 -> 620 (4), 1280 870 -> 771 (5), 1664 1171 -> 1036 (4), 2048
+// 1204 -> 1213 (stays with score.cu); d = 1024, V = 64000: 300 52.8 -> 41.5 (2), 448 54.4 -> 50.3 (2), 512 55.4 -> 54.8
+// (2); d = 512, V = 32000: 384 24.0 -> 23.2 (2), 448 24.1 -> 24.5 (stays); d = 256, V = 64000: 384 26.0 -> 29.3 (stays).
+// Up to 256 rows (one row block) both kernels follow the W stream.  This one wins where score.cu's mostly
+// empty boxes of H hold it up (N = 32, d = 1024 38.0 -> 30.4; N = 64 30.2 -> 30.9) and where the W stream is long
+// enough for the power limit to bite (d = 3072, V = 126464, N = 128 129 -> 119; d = 4096 168 -> 154, N = 208 175 -> 171,
+// N = 256 183 -> 190; but d = 2048, V = 64000, N = 128 49.6 -> 50.3).
+constexpr int kVmShortRows = 48;                        // always here (with a vocabulary for every pair's records)
+constexpr int64_t kVmLongHead = int64_t(1) << 28;       // V * d from which one row block may come here, 512 MiB of W
+constexpr int64_t kRowOneBlockSliceNs = 350;            // a K slice of score.cu's tile of a single row block there
 constexpr int kVmMaxGroups = 8;
 constexpr int kVmEvenTileRows = 192;  // rows per group up to which the W stream, not the MMAs, sets the time: tiles are
                                       // then narrowed to split the vocabulary evenly over the pairs (V = 126464 on 76
@@ -461,7 +466,7 @@ namespace {
 // The split over n_groups row groups: each group of pairs owns hw[0] + hw[1] consecutive rows of H and, as in
 // score.cu, walks the vocabulary tiles side by side.  Two records per pair (one per CTA) and row.  False when it
 // cannot run with that many groups.
-bool vm_split(int64_t N, int64_t V, int max_units, int32_t records_cap, int32_t n_groups, VmSchedule *out)
+bool vm_split(int64_t N, int64_t n_kb, int64_t V, int max_units, int32_t records_cap, int32_t n_groups, VmSchedule *out)
 {
     VmSchedule s{};
     const int64_t rows = (N + n_groups - 1) / n_groups;
@@ -489,7 +494,9 @@ bool vm_split(int64_t N, int64_t V, int max_units, int32_t records_cap, int32_t 
     s.bn = (int32_t)bn;
     s.n_vt = (int32_t)((V + bn - 1) / bn);
     s.G = (int32_t)(g < s.n_vt ? g : s.n_vt);
-    s.cost = tiles * (s.hw[1] > 0 ? 75 + (s.hw[0] + s.hw[1]) * 7 / 5 : 130 + s.hw[0]);
+    const int64_t w = s.hw[0] + s.hw[1], epilogue = 15 * w;
+    s.cost = epilogue + tiles * (s.hw[1] > 0 ? n_kb * (60 + w * 7 / 5) + 4 * w
+                                             : (n_kb * (130 + w) > epilogue ? n_kb * (130 + w) : epilogue));
     s.stage_bytes = kVmStageBytesW + (uint32_t)((s.hw[0] + s.hw[1]) / 2) * 128u;
     const uint32_t fit = kVmRingCapacity / s.stage_bytes;
     s.stages = (int32_t)(fit < (uint32_t)kVmMaxStages ? fit : (uint32_t)kVmMaxStages);
@@ -502,19 +509,23 @@ bool vm_split(int64_t N, int64_t V, int max_units, int32_t records_cap, int32_t 
 bool score_vmajor_schedule(int64_t N, int64_t d, int64_t V, int max_units, int32_t records_cap,
                            const ScoreSchedule &rows, VmSchedule *out)
 {
+    const int64_t n_kb = (d + kBK - 1) / kBK;
     bool found = false;
-    for (int32_t g = 1; g <= kVmMaxGroups; ++g) {
+    const int32_t most = N <= kPairM ? 1 : kVmMaxGroups;  // one row block is bound by the W stream: no second reader
+    for (int32_t g = 1; g <= most; ++g) {
         VmSchedule s;
-        if (vm_split(N, V, max_units, records_cap, g, &s) && (!found || s.cost < out->cost)) {
+        if (vm_split(N, n_kb, V, max_units, records_cap, g, &s) && (!found || s.cost < out->cost)) {
             *out = s;
             found = true;
         }
     }
-    if (!found || ((d + kBK - 1) / kBK < kVmMinSlices && N > kVmShortRows))
-        return false;
+    if (!found || N <= kVmShortRows)
+        return found;
     const int64_t blocks = (N + kPairM - 1) / kPairM;
     const int64_t row_tiles = (blocks + rows.n_groups - 1) / rows.n_groups * ((rows.n_vt + rows.G - 1) / rows.G);
-    return out->cost < row_tiles * (blocks == 1 ? kRowTileCostOneBlock : kRowTileCost);
+    if (blocks == 1)
+        return V * d >= kVmLongHead && out->cost < row_tiles * n_kb * kRowOneBlockSliceNs;
+    return out->cost < row_tiles * (n_kb * 380 + 700);
 }
 
 cudaError_t launch_score_vmajor(const CUtensorMap &tmH, const CUtensorMap &tmW, const ScoreArgs &a, bool entropy,

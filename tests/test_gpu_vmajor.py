@@ -17,16 +17,15 @@ pytestmark = pytest.mark.gpu
 SHAPES = [
     (1, 8, 19456, 1 * 76),         # one row, one K slice (mostly zero fill), one 32-column chunk
     (33, 72, 20001, 1 * 139),      # 64 columns, K tail, 144-wide tiles, the last one mostly past the vocabulary
-    (64, 256, 40000, 1 * 228),     # 176-wide tiles
-    (97, 1536, 19456, 1 * 76),     # 128 columns, 31 of them padding
-    (129, 1544, 19500, 1 * 136),   # one accumulator of 144 columns: a half chunk at its end
-    (200, 1536, 23001, 1 * 90),    # 208 columns, 256-wide tiles
-    (257, 1536, 19456, 1 * 76),    # 144 + 128 columns, three accumulators in TMEM
+    (48, 256, 40000, 1 * 228),     # 176-wide tiles
+    (257, 1536, 19456, 2 * 76),    # two groups of one accumulator of 144 columns: a half chunk at its end
     (300, 1600, 19457, 2 * 77),    # two groups of 160 columns, a last tile of one vocabulary entry
-    (432, 1536, 19456, 1 * 76),    # 224 + 208 columns, two accumulators in TMEM
-    (577, 1536, 19456, 2 * 76),    # two groups of 304 rows, the second ragged
+    (340, 1024, 19500, 2 * 77),    # 176 columns
+    (400, 1536, 19456, 2 * 76),    # 208 columns
+    (300, 4096, 19456, 1 * 76),    # 160 + 144 columns, three accumulators in TMEM
+    (330, 3072, 19456, 1 * 76),    # 176 + 160 columns, two accumulators in TMEM
+    (530, 1024, 26112, 2 * 102),   # two groups of 144 + 128 columns, the second ragged
     (960, 1536, 19456, 4 * 76),    # four groups of one accumulator of 240 columns
-    (1100, 1536, 19456, 4 * 76),   # four groups of 144 + 144 columns, the last one ragged
 ]
 
 
