@@ -39,9 +39,12 @@ constexpr int kVmThreads = 64 + 32 * kVmEpiWarps;
 constexpr int kMaxChunks = 4;  // 32-column chunks of one accumulator (256 columns) per epilogue warp
 // The split and the choice between the two score kernels: ns on the busiest pair, fitted to steps in steady state
 // (d = 4096, V = 126464, N from 128 to 2048, 1 to 8 groups; d = 256 to 1536 with V from 20000 to 64000; within 5 % of
-// most).  Per tile: n_kb K slices of 130 + hw with one accumulator, or the epilogue (15 ns a column) if that is longer,
-// as the accumulators alternate; 60 + 1.4 (hw[0] + hw[1]) with two, and part of their epilogue (4 ns a column).  Then
-// the last tile's epilogue.  score.cu: 380 per K slice of a 256-row tile, and 700 for its epilogue.
+// most).  Per tile: n_kb K slices of 190 + 0.75 hw with one accumulator (each SM receives 85 GB/s of W and H), of 60 + 1.4 (hw[0] + hw[1]) with two and 4 ns a
+// column for their epilogue's exposed part, or the epilogue (992 ns for two 32-column chunks, one per warp) if that is
+// longer.  Then the last tile's epilogue.  score.cu: per tile 380 per K slice at bn = 256 (narrower MMAs save less than their columns)
+// and 700 for its epilogue, or the epilogue alone (9.7 ns a column) if that is longer, and the last tile's epilogue.
+// On 70 random shapes (N to 2048, d to 4096, V from 19456) the choice was within 4 % of the best split of either kernel
+// on 65, and at worst 12 % off it and 7 % slower than score.cu.
 // us per step, score.cu -> here (groups), d = 4096, V = 126464: N = 288 308 -> 220 (1), 320 316 -> 243 (1),
 // 384 326 -> 287 (1, 2), 448 333 -> 312 (2), 512 344 -> 346 (2), 576 494 -> 390 (2), 640 502 -> 421 (2),
 // 768 523 -> 482 (3), 896 616 -> 578 (4), 1024 632 -> 620 (4), 1280 870 -> 771 (5), 1664 1171 -> 1036 (4), 2048
@@ -52,8 +55,9 @@ constexpr int kMaxChunks = 4;  // 32-column chunks of one accumulator (256 colum
 // enough for the power limit to bite (d = 3072, V = 126464, N = 128 129 -> 119; d = 4096 168 -> 154, N = 208 175 -> 171,
 // N = 256 183 -> 190; but d = 2048, V = 64000, N = 128 49.6 -> 50.3).
 constexpr int kVmShortRows = 48;                        // always here (with a vocabulary for every pair's records)
+constexpr int kVmMinSlices = 4;                         // K slices per tile: below, latencies that the estimates leave out
 constexpr int64_t kVmLongHead = int64_t(1) << 28;       // V * d from which one row block may come here, 512 MiB of W
-constexpr int64_t kRowOneBlockSliceNs = 350;            // a K slice of score.cu's tile of a single row block there
+constexpr int64_t kRowOneBlockSliceNs = 356;            // a K slice of score.cu's tile of a single row block there
 constexpr int kVmMaxGroups = 8;
 constexpr int kVmEvenTileRows = 192;  // rows per group up to which the W stream, not the MMAs, sets the time: tiles are
                                       // then narrowed to split the vocabulary evenly over the pairs (V = 126464 on 76
@@ -494,9 +498,10 @@ bool vm_split(int64_t N, int64_t n_kb, int64_t V, int max_units, int32_t records
     s.bn = (int32_t)bn;
     s.n_vt = (int32_t)((V + bn - 1) / bn);
     s.G = (int32_t)(g < s.n_vt ? g : s.n_vt);
-    const int64_t w = s.hw[0] + s.hw[1], epilogue = 15 * w;
-    s.cost = epilogue + tiles * (s.hw[1] > 0 ? n_kb * (60 + w * 7 / 5) + 4 * w
-                                             : (n_kb * (130 + w) > epilogue ? n_kb * (130 + w) : epilogue));
+    const int64_t w = s.hw[0] + s.hw[1], chunks = (s.hw[0] + 31) / 32 + (s.hw[1] + 31) / 32;
+    const int64_t mma = s.hw[1] > 0 ? n_kb * (60 + w * 7 / 5) + 4 * w : n_kb * (190 + w * 3 / 4);
+    const int64_t epilogue = (chunks + 1) / 2 * 992;
+    s.cost = epilogue + tiles * (mma > epilogue ? mma : epilogue);
     s.stage_bytes = kVmStageBytesW + (uint32_t)((s.hw[0] + s.hw[1]) / 2) * 128u;
     const uint32_t fit = kVmRingCapacity / s.stage_bytes;
     s.stages = (int32_t)(fit < (uint32_t)kVmMaxStages ? fit : (uint32_t)kVmMaxStages);
@@ -523,9 +528,12 @@ bool score_vmajor_schedule(int64_t N, int64_t d, int64_t V, int max_units, int32
         return found;
     const int64_t blocks = (N + kPairM - 1) / kPairM;
     const int64_t row_tiles = (blocks + rows.n_groups - 1) / rows.n_groups * ((rows.n_vt + rows.G - 1) / rows.G);
+    if (n_kb < kVmMinSlices)
+        return false;
     if (blocks == 1)
         return V * d >= kVmLongHead && out->cost < row_tiles * n_kb * kRowOneBlockSliceNs;
-    return out->cost < row_tiles * (n_kb * 380 + 700);
+    const int64_t mma = n_kb * 380 * (rows.bn + 144) / 400 + 700, epilogue = 97 * rows.bn / 10;
+    return out->cost < row_tiles * (mma > epilogue ? mma : epilogue) + epilogue;
 }
 
 cudaError_t launch_score_vmajor(const CUtensorMap &tmH, const CUtensorMap &tmW, const ScoreArgs &a, bool entropy,

@@ -18,14 +18,13 @@ SHAPES = [
     (1, 8, 19456, 1 * 76),         # one row, one K slice (mostly zero fill), one 32-column chunk
     (33, 72, 20001, 1 * 139),      # 64 columns, K tail, 144-wide tiles, the last one mostly past the vocabulary
     (48, 256, 40000, 1 * 228),     # 176-wide tiles
-    (257, 1536, 19456, 2 * 76),    # two groups of one accumulator of 144 columns: a half chunk at its end
-    (300, 1600, 19457, 2 * 77),    # two groups of 160 columns, a last tile of one vocabulary entry
-    (340, 1024, 19500, 2 * 77),    # 176 columns
-    (400, 1536, 19456, 2 * 76),    # 208 columns
-    (300, 4096, 19456, 1 * 76),    # 160 + 144 columns, three accumulators in TMEM
-    (330, 3072, 19456, 1 * 76),    # 176 + 160 columns, two accumulators in TMEM
-    (530, 1024, 26112, 2 * 102),   # two groups of 144 + 128 columns, the second ragged
-    (960, 1536, 19456, 4 * 76),    # four groups of one accumulator of 240 columns
+    (257, 512, 24118, 3 * 95),     # three groups of one accumulator of 96 columns, the last one ragged
+    (257, 512, 25672, 2 * 101),    # 144 columns: a half chunk at the accumulator's end
+    (257, 512, 38881, 1 * 152),    # 144 + 128 columns, three accumulators in TMEM
+    (327, 1544, 29557, 1 * 116),   # 176 + 160 columns, two accumulators in TMEM
+    (390, 1024, 24118, 2 * 95),    # 208 columns
+    (530, 1024, 25672, 2 * 101),   # two groups of 144 + 128 columns, the second ragged
+    (726, 1024, 24118, 3 * 95),    # 256 columns
 ]
 
 
