@@ -1,22 +1,22 @@
 // finish.cu -- the end of a WINO step (sm_103a): merge the score kernel's
 // partial softmax records per row, then apply Eq. 4 to the token state.
 //
-// finish_kernel: one warp per row folds the row's G partial records (fixed
-// lane order, then a butterfly, so results are bit-for-bit reproducible) into
+// One warp per row folds the row's partial records (fixed lane order, then a butterfly, so results are bit-for-bit
+// reproducible) into
 //   argmax   = smallest vocabulary id among the maximal logits,
 //   pmax     = max_v p_v = 1 / sum_v exp(l_v - m),
 //   ptarget  = p_target = exp(l_t - m) / sum_v exp(l_v - m)    (0 without a target),
 // the three statistics Eq. 2 and Eq. 3 use, and on request the entropy
 //   H(p)     = -sum_v p_v log p_v = ln Z - sum_v exp(l_v - m) (l_v - m) / Z
-// that WINO+'s deferral and sharpening terms use (Sec. 5.3, Eq. 6-7).  In a whole step (wino_step) every
-// CTA then adds its merged rows to its sequences' tickets; the CTA that
-// completes a sequence's 2*L_b rows applies Eq. 4 to that sequence, so merge
-// and update need one launch.  Tickets are cleared by the score kernel of the
-// same step.  The kernel is launched programmatically: its CTAs start beside the
-// score kernel's and wait (griddepcontrol.wait) for the score kernel's
-// results before touching them; it lets the next call's kernels launch at once
-// (they only prefetch W before their own griddepcontrol.wait).  The last of
-// its CTAs to merge its rows publishes the call's status (see StatusWords).
+// that WINO+'s deferral and sharpening terms use (Sec. 5.3, Eq. 6-7).  In a whole step (wino_step) Eq. 4 follows in
+// the same launch:
+//   finish_step_kernel, sequences of up to 128 rows: a cluster of CTAs per sequence merges its rows and hands the
+//     statistics to its first CTA, which applies Eq. 4;
+//   finish_kernel, longer sequences: every CTA adds its merged rows to its sequences' tickets (cleared by the score
+//     kernel of the same step), and the CTA that completes a sequence applies Eq. 4.
+// Both are launched programmatically: their CTAs start beside the score kernel's and wait (griddepcontrol.wait) for
+// its results before touching them; they let the next call's kernels launch at once (those only prefetch W before
+// their own griddepcontrol.wait).  They publish the call's status (see StatusWords).
 //
 // draft_verify_kernel: Eq. 4 alone from caller-supplied statistics
 // (wino_draft_verify), one CTA per sequence.
@@ -34,6 +34,8 @@
 // is applied in place in one pass after a CTA-wide reduction.  With
 // WINO_OPT_FREEZE_FINISHED a sequence whose block already has no MASK is left
 // as it is (its own loop, Sec. 4.2.3, has ended).
+#include <algorithm>
+
 #include "fold.cuh"
 #include "internal.h"
 #include "ptx.cuh"
@@ -43,6 +45,7 @@ namespace {
 
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr int kFinishRows = 8;  // rows (warps) per finish CTA; also the CTA size of the Eq. 4 kernels
+constexpr int kClusterSeqRows = 128;  // rows of a sequence up to which a cluster of CTAs finishes it: two rows per warp
 constexpr int kRecInFlight = 5;  // records each lane loads at once (160 per row: two per pair of a 76-pair launch fit)
 
 // Block-wide reduction scratch for eq4_block.
@@ -56,16 +59,44 @@ struct Eq4Smem {
 extern __shared__ float s_conf[];
 inline uint32_t conf_bytes(const wino_params &p) { return p.draft_m > 0 ? (uint32_t)p.blk_len * 4u : 0u; }
 
-// Eq. 4 on sequence s by the whole CTA (kFinishRows warps; thread t owns positions t, t + 256, ...),
-// reading the statistics of the a-th sequence of the scored rows (a = s unless an active-sequence list
-// chose the rows).  Every load is issued before any decision so the update costs about one memory round
-// trip.  Statistics are read through L2: other CTAs of the same launch may have written them.
-__device__ void eq4_block(int a, int s, int32_t *tokens, const int32_t *argmax, const float *pmax,
-                          const float *ptarget, const wino_params &p, int32_t *counts, int8_t *flags, int32_t status,
-                          Eq4Smem &sm)
+constexpr int kEq4Threads = kFinishRows * 32;
+constexpr int kEq4Per = kMaxBlkLen / kEq4Threads;  // positions per thread
+
+// Where Eq. 4 finds a sequence's statistics: entry l of argmax and pmax belongs to the row read for a masked position
+// l, entry l of ptarget to the row read for a decoded one.
+struct SeqStats {
+    const int32_t *argmax;
+    const float *pmax, *ptarget;
+};
+
+// The same from per-row arrays whose first row of the sequence is row `first`.
+__device__ __forceinline__ SeqStats seq_stats(const int32_t *argmax, const float *pmax, const float *ptarget,
+                                              int64_t first, const wino_params &p)
 {
-    constexpr int kT = kFinishRows * 32;
-    constexpr int kPer = kMaxBlkLen / kT;
+    const bool both = !(p.options & (WINO_OPT_NO_SHADOW | WINO_OPT_COMPACT));  // block rows, then shadow rows
+    return SeqStats{argmax + first, pmax + first, ptarget ? ptarget + first + (both ? p.blk_len : 0) : nullptr};
+}
+
+// The current tokens of sequence s's block, thread t's positions t, t + 256, ...
+__device__ __forceinline__ void load_tokens(const int32_t *tokens, int s, const wino_params &p, int32_t (&yv)[kEq4Per])
+{
+    const int32_t *y = tokens + (int64_t)s * p.seq_len + p.blk_start;
+#pragma unroll
+    for (int i = 0; i < kEq4Per; ++i) {
+        const int l = (int)threadIdx.x + i * kEq4Threads;
+        yv[i] = l < p.blk_len ? y[l] : 0;
+    }
+}
+
+// Eq. 4 on sequence s, whose block holds the tokens yv, by the whole CTA.  Every load is issued before any decision so
+// the update costs about one memory round trip.  kShared: the statistics are in this CTA's shared memory; otherwise
+// they are read through L2, as other CTAs of the same launch may have written them.
+template <bool kShared>
+__device__ void eq4_block(int s, const int32_t (&yv)[kEq4Per], const SeqStats st, int32_t *tokens, const wino_params &p,
+                          int32_t *counts, int8_t *flags, int32_t status, Eq4Smem &sm)
+{
+    constexpr int kT = kEq4Threads;
+    constexpr int kPer = kEq4Per;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (status != WINO_OK) {  // the scores of this step are invalid: leave the state alone
         if (tid < 3)
@@ -75,21 +106,18 @@ __device__ void eq4_block(int a, int s, int32_t *tokens, const int32_t *argmax, 
     const int L = p.blk_len;
     const int32_t mask = p.mask_id;
     const bool shadow = !(p.options & WINO_OPT_NO_SHADOW);  // WINO+ inference has no verification rows
-    const bool compact = (p.options & WINO_OPT_COMPACT) != 0;  // one row per position
     int32_t *y = tokens + (int64_t)s * p.seq_len + p.blk_start;
-    const int64_t rb = (int64_t)((shadow && !compact) ? 2 * a : a) * L;  // rows read for masked positions
-    const int64_t rs = (int64_t)(compact ? a : 2 * a + 1) * L;         // rows read for decoded positions
 
-    int32_t yv[kPer], av[kPer];
+    int32_t av[kPer];
     float pm[kPer], pt[kPer];
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
         const int l = tid + i * kT;
         if (l < L) {
-            yv[i] = y[l];
-            av[i] = __ldcg(argmax + rb + l);
-            pm[i] = __ldcg(pmax + rb + l);
-            pt[i] = shadow ? __ldcg(ptarget + rs + l) : 1.0f;  // 1.0 is never below tau2 <= 1: no re-mask
+            av[i] = kShared ? st.argmax[l] : __ldcg(st.argmax + l);
+            pm[i] = kShared ? st.pmax[l] : __ldcg(st.pmax + l);
+            // 1.0 is never below tau2 <= 1: no re-mask
+            pt[i] = !shadow ? 1.0f : (kShared ? st.ptarget[l] : __ldcg(st.ptarget + l));
         }
     }
     // Pass 1: how many masked positions clear tau1, and the most confident masked position.
@@ -228,23 +256,183 @@ __device__ void eq4_block(int a, int s, int32_t *tokens, const int32_t *argmax, 
     __syncthreads();  // the scratch may be reused for the next sequence
 }
 
-// The status that invalidates this call's scores (WINO_ERR_ARG is the finish kernel's own, see bad_entry).
-__device__ __forceinline__ int32_t score_status(const StatusWords *w)
-{
-    const int32_t s = *reinterpret_cast<const volatile int32_t *>(&w->current);
-    return s == WINO_ERR_ARG ? (int32_t)WINO_OK : s;
-}
-
 // Whether the caller's active-sequence list names no sequence of the batch for the a-th scored sequence.
 __device__ __forceinline__ bool bad_entry(const wino_params &p, int64_t a)
 {
     return p.active_seq && (p.active_seq[a] < 0 || p.active_seq[a] >= p.n_seq);
 }
 
-// Eq. 4: the CTA that merges the last rows of a sequence updates that sequence.
-__device__ void eq4_tail(const FinishArgs &a, int64_t row0, int64_t per_seq, int32_t status, int32_t *s_done,
-                         int32_t &s_ndone, Eq4Smem &sm)
+// A row's merged softmax state.
+struct Merged {
+    float m, s, tl, u;
+    int32_t idx;
+};
+
+// Merge the records of rows row[0 .. kU) (negative: no row) by a warp, kK records per row, lane and round in flight.
+// Fixed lane order, then a butterfly.  The record of the pair whose tiles hold the row's target carries its logit, the
+// others -inf.
+template <int kU, int kK, bool kEntropy>
+__device__ __forceinline__ void merge_rows(const FinishArgs &a, const int64_t (&row)[kU], Merged (&o)[kU])
 {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+        o[u] = Merged{-INFINITY, 0.f, -INFINITY, 0.f, INT32_MAX};
+    for (int j0 = 0; j0 < a.G; j0 += 32 * kK) {
+        float4 r[kU][kK];
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+#pragma unroll
+            for (int i = 0; i < kK; ++i) {
+                const int j = j0 + lane + 32 * i;
+                r[u][i] = (row[u] >= 0 && j < a.G) ? __ldcg(a.part + row[u] * a.G + j)
+                                                   : make_float4(-INFINITY, 0.f, __int_as_float(INT32_MAX), -INFINITY);
+            }
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+#pragma unroll
+            for (int i = 0; i < kK; ++i) {
+                const int j = j0 + lane + 32 * i;
+                if (kEntropy)
+                    combine_u(o[u].m, o[u].s, o[u].u, o[u].idx, r[u][i].x, r[u][i].y,
+                              (row[u] >= 0 && j < a.G) ? __ldcg(a.part_u + row[u] * a.G + j) : 0.f,
+                              __float_as_int(r[u][i].z));
+                else
+                    combine(o[u].m, o[u].s, o[u].idx, r[u][i].x, r[u][i].y, __float_as_int(r[u][i].z));
+                o[u].tl = fmaxf(o[u].tl, r[u][i].w);
+            }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const float m2 = __shfl_xor_sync(0xffffffffu, o[u].m, off);
+            const float s2 = __shfl_xor_sync(0xffffffffu, o[u].s, off);
+            const int32_t i2 = __shfl_xor_sync(0xffffffffu, o[u].idx, off);
+            o[u].tl = fmaxf(o[u].tl, __shfl_xor_sync(0xffffffffu, o[u].tl, off));
+            if (kEntropy)
+                combine_u(o[u].m, o[u].s, o[u].u, o[u].idx, m2, s2, __shfl_xor_sync(0xffffffffu, o[u].u, off), i2);
+            else
+                combine(o[u].m, o[u].s, o[u].idx, m2, s2, i2);
+        }
+}
+
+// The three statistics of a merged row; invalid ones (status != WINO_OK) are -1 and NaN.
+struct RowStats {
+    int32_t argmax;
+    float pmax, ptarget;
+};
+__device__ __forceinline__ RowStats row_stats(const Merged &o, int32_t status)
+{
+    if (status != WINO_OK)
+        return RowStats{-1, __int_as_float(0x7fc00000), __int_as_float(0x7fc00000)};
+    return RowStats{o.idx, 1.0f / o.s, (o.tl > -INFINITY) ? ptx::ex2((o.tl - o.m) * kLog2e) / o.s : 0.0f};
+}
+
+__device__ __forceinline__ void store_row(const FinishArgs &a, int64_t row, const RowStats &x)
+{
+    a.argmax[row] = x.argmax;
+    a.pmax[row] = x.pmax;
+    a.ptarget[row] = x.ptarget;
+}
+
+// Publish the call's outcome; every thread of every CTA calls it with the `current` word it read.  Without a failure
+// nobody writes that word, and the first CTA stores the outcome (a bad active-sequence entry is the only error left).
+// After a failure the last CTA to come here also clears the word, which every CTA has then read.
+__device__ __forceinline__ void publish_status(const FinishArgs &a, int32_t status, int64_t n_scored_seq)
+{
+    if (status == WINO_OK) {
+        if (blockIdx.x == 0 && threadIdx.x < 32) {
+            bool bad = false;
+            if (a.tokens && a.p.active_seq)
+                for (int64_t i = threadIdx.x; i < n_scored_seq; i += 32)
+                    bad |= bad_entry(a.p, i);
+            bad = __any_sync(0xffffffffu, bad);
+            if (threadIdx.x == 0)
+                a.status->last = bad ? (int32_t)WINO_ERR_ARG : (int32_t)WINO_OK;
+        }
+        return;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&a.status->finished, 1u) == gridDim.x - 1) {
+        __threadfence();
+        a.status->finished = 0;
+        a.status->last = atomicExch(&a.status->current, (int32_t)WINO_OK);
+    }
+}
+
+// The end of a step whose sequences have at most kClusterSeqRows rows: a cluster of up to 8 CTAs per sequence.  Its
+// warps merge the sequence's rows and hand the statistics to the first CTA's shared memory; behind one cluster barrier
+// that CTA applies Eq. 4, whose tokens it has loaded meanwhile.
+// What bounds it is latency: dependent round trips to L2 and barriers after the score kernel's last CTA.  The CTAs are
+// small enough in registers and shared memory to start beside most score CTAs and wait there (with 64 registers and
+// 4.3 KB of shared memory they started only when score CTAs left: 9.5 -> 8.5 us for the tiny step in a CUDA graph).
+// Handing over through global memory (finish_kernel: one CTA per 8 rows, fences, a ticket per sequence, the statistics
+// read back) costs about 3 us more, but merges more rows at once.  us per step, finish_kernel -> here: 64 rows 9.2 ->
+// 7.9 (d = 64, V = 1000), 151.0 -> 147.8 (d = 4096, V = 126464); 128 rows 9.3 -> 8.5; 256 rows 12.2 -> 13.0 and 512 rows
+// 10.3 -> 13.4, so longer sequences stay with finish_kernel.
+__global__ void __launch_bounds__(kFinishRows * 32, 5) finish_step_kernel(const FinishArgs a)
+{
+    ptx::grid_dep_launch_dependents();  // the next call may start streaming its H and W
+    __shared__ Eq4Smem sm;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = ptx::cluster_ctarank();
+    const int seq = (int)blockIdx.x / a.cluster, R = a.seq_rows;
+    // dynamic shared memory: [fixed-M scratch | argmax[R] | pmax[R] | ptarget[R]]
+    int32_t *s_argmax = reinterpret_cast<int32_t *>(s_conf + (a.p.draft_m > 0 ? a.p.blk_len : 0));
+    float *s_pmax = reinterpret_cast<float *>(s_argmax + R), *s_ptarget = s_pmax + R;
+    ptx::cluster_sync();  // the first CTA has started: its shared memory may be written
+    ptx::grid_dep_wait();
+    const int32_t status = *reinterpret_cast<const volatile int32_t *>(&a.status->current);
+    int32_t yv[kEq4Per];
+    int s = -1;
+    if (rank == 0 && !bad_entry(a.p, seq)) {
+        s = a.p.active_seq ? a.p.active_seq[seq] : seq;
+        load_tokens(a.tokens, s, a.p, yv);
+    }
+    const int64_t first = (int64_t)seq * R;
+    const int stride = a.cluster * kFinishRows;
+    auto hand_over = [&](int r, const Merged &o) {  // row r of the sequence, by lane 0
+        const RowStats x = row_stats(o, status);
+        store_row(a, first + r, x);
+        ptx::st_shared_cluster_u32(ptx::mapa(ptx::smem_u32(s_argmax + r), 0), (uint32_t)x.argmax);
+        ptx::st_shared_cluster_u32(ptx::mapa(ptx::smem_u32(s_pmax + r), 0), __float_as_uint(x.pmax));
+        ptx::st_shared_cluster_u32(ptx::mapa(ptx::smem_u32(s_ptarget + r), 0), __float_as_uint(x.ptarget));
+    };
+    int r = (int)rank * kFinishRows + warp;
+    if (R <= stride) {  // one row per warp
+        if (r < R) {
+            Merged o[1];
+            merge_rows<1, kRecInFlight, false>(a, {first + r}, o);
+            if (lane == 0)
+                hand_over(r, o[0]);
+        }
+    } else {
+        for (; r < R; r += 2 * stride) {
+            const int r2 = r + stride;
+            Merged o[2];
+            merge_rows<2, 3, false>(a, {first + r, r2 < R ? first + r2 : -1}, o);
+            if (lane == 0) {
+                hand_over(r, o[0]);
+                if (r2 < R)
+                    hand_over(r2, o[1]);
+            }
+        }
+    }
+    __syncwarp();
+    ptx::cluster_sync();  // the statistics are in the first CTA's shared memory
+    if (s >= 0)
+        eq4_block<true>(s, yv, seq_stats(s_argmax, s_pmax, s_ptarget, 0, a.p), a.tokens, a.p, a.counts, a.flags, status,
+                        sm);
+    publish_status(a, status, a.N / R);
+}
+
+// Eq. 4 at the end of finish_kernel: the CTA that merges the last rows of a sequence updates that sequence.
+__device__ void eq4_tail(const FinishArgs &a, int64_t row0, int32_t status, int32_t *s_done, int32_t &s_ndone,
+                         Eq4Smem &sm)
+{
+    __syncthreads();
+    const int64_t per_seq = a.seq_rows;
     if (threadIdx.x == 0) {
         int32_t nd = 0;
         const int64_t rend = min(row0 + kFinishRows, (int64_t)a.N);
@@ -262,90 +450,48 @@ __device__ void eq4_tail(const FinishArgs &a, int64_t row0, int64_t per_seq, int
     __syncthreads();
     const int nd = s_ndone;
     for (int i = 0; i < nd; ++i) {
-        if (bad_entry(a.p, s_done[i]))
+        const int sq = s_done[i];
+        if (bad_entry(a.p, sq))
             continue;  // no update (the status says so)
-        const int sq = a.p.active_seq ? a.p.active_seq[s_done[i]] : s_done[i];
-        eq4_block(s_done[i], sq, a.tokens, a.argmax, a.pmax, a.ptarget, a.p, a.counts, a.flags, status, sm);
+        const int s = a.p.active_seq ? a.p.active_seq[sq] : sq;
+        int32_t yv[kEq4Per];
+        load_tokens(a.tokens, s, a.p, yv);
+        eq4_block<false>(s, yv, seq_stats(a.argmax, a.pmax, a.ptarget, sq * per_seq, a.p), a.tokens, a.p, a.counts,
+                         a.flags, status, sm);
     }
 }
 
-// What bounds it is latency: a chain of dependent round trips to L2 (records; tickets; statistics) after the score
-// kernel's last CTA.  Its CTAs are small enough in registers and shared memory to be resident beside the score CTAs
-// and wait there, the records are loaded without waiting for the status word, and the count of finished CTAs runs
-// beside the tickets and Eq. 4.  With 64 registers a thread and 4.3 KB of shared memory it started only when score CTAs
-// left their SMs.  us per step in a CUDA graph, before -> after: d = 64, V = 1000, N = 64 9.5 -> 8.5; d = 512,
-// V = 32000, N = 128 14.3 -> 13.3; d = 1024, V = 64000, N = 256 30.0 -> 29.2; nothing measurable from 150 us up.
+// Rows without a state update (wino_score_rows), and the end of a step with longer sequences: one warp per row.  As
+// finish_step_kernel, it is bound by latency; without a state update it neither fences nor counts its CTAs (333 rows at
+// d = 1024, V = 32000: 28.2 -> 26.5 us per call).
 __global__ void __launch_bounds__(kFinishRows * 32, 5) finish_kernel(const FinishArgs a)
 {
     ptx::grid_dep_launch_dependents();  // the next call may start streaming its H and W
     __shared__ int32_t s_done[kFinishRows];
     __shared__ int32_t s_ndone;
     __shared__ Eq4Smem sm;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t row0 = (int64_t)blockIdx.x * kFinishRows;
-    const int64_t row = row0 + warp;
-    const int64_t per_seq =
-        ((a.p.options & (WINO_OPT_NO_SHADOW | WINO_OPT_COMPACT)) ? 1 : 2) * (int64_t)a.p.blk_len;  // rows
+    const int64_t row = row0 + (threadIdx.x >> 5);
     ptx::grid_dep_wait();
-    const int32_t status = score_status(a.status);
-
+    const int32_t status = *reinterpret_cast<const volatile int32_t *>(&a.status->current);
     if (row < a.N) {
-        // Every record of the row (the workspace holds them whatever the status); the record of the pair whose tiles
-        // hold the row's target carries its logit, the others -inf.
-        const float4 *pr = a.part + row * a.G;
-        float m = -INFINITY, s = 0.f, tl = -INFINITY, u = 0.f;
-        int32_t idx = INT32_MAX;
-        for (int j0 = 0; j0 < a.G; j0 += 32 * kRecInFlight) {
-            float4 r[kRecInFlight];
-#pragma unroll
-            for (int i = 0; i < kRecInFlight; ++i) {
-                const int j = j0 + lane + 32 * i;
-                r[i] = (j < a.G) ? __ldcg(pr + j) : make_float4(-INFINITY, 0.f, __int_as_float(INT32_MAX), -INFINITY);
-            }
-#pragma unroll
-            for (int i = 0; i < kRecInFlight; ++i) {
-                const int j = j0 + lane + 32 * i;
-                if (!a.entropy)
-                    combine(m, s, idx, r[i].x, r[i].y, __float_as_int(r[i].z));
-                else
-                    combine_u(m, s, u, idx, r[i].x, r[i].y,
-                              (j < a.G) ? __ldcg(a.part_u + row * a.G + j) : 0.f, __float_as_int(r[i].z));
-                tl = fmaxf(tl, r[i].w);
-            }
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-            const float s2 = __shfl_xor_sync(0xffffffffu, s, off);
-            const int32_t i2 = __shfl_xor_sync(0xffffffffu, idx, off);
-            tl = fmaxf(tl, __shfl_xor_sync(0xffffffffu, tl, off));
-            if (!a.entropy)
-                combine(m, s, idx, m2, s2, i2);
-            else
-                combine_u(m, s, u, idx, m2, s2, __shfl_xor_sync(0xffffffffu, u, off), i2);
-        }
-        if (lane == 0) {
-            const bool ok = status == WINO_OK;
-            const float nan = __int_as_float(0x7fc00000);
-            a.argmax[row] = ok ? idx : -1;
-            a.pmax[row] = ok ? 1.0f / s : nan;
-            a.ptarget[row] = !ok ? nan : ((tl > -INFINITY) ? ptx::ex2((tl - m) * kLog2e) / s : 0.0f);
+        Merged o[1];
+        if (a.entropy)
+            merge_rows<1, kRecInFlight, true>(a, {row}, o);
+        else
+            merge_rows<1, kRecInFlight, false>(a, {row}, o);
+        if ((threadIdx.x & 31) == 0) {
+            store_row(a, row, row_stats(o[0], status));
             if (a.entropy)  // H = ln Z - (u ln 2) / Z, with u in log2 units
-                a.entropy[row] = ok ? (ptx::lg2(s) - u / s) * kLn2 : nan;
-            if (a.tokens && bad_entry(a.p, row / per_seq))  // reported unless the scores already failed
-                atomicCAS(&a.status->current, (int32_t)WINO_OK, (int32_t)WINO_ERR_ARG);
-            __threadfence();  // publish this row and the status before the CTA signals its ticket and its end
+                a.entropy[row] = status == WINO_OK ? (ptx::lg2(o[0].s) - o[0].u / o[0].s) * kLn2
+                                                   : __int_as_float(0x7fc00000);
+            if (a.tokens)
+                __threadfence();  // publish this row before the CTA signals its ticket
         }
-    }
-    __syncthreads();
-    // The last CTA to come here publishes the call's status and clears the word for the next call: every CTA has read
-    // the word, and recorded its own errors, before.
-    if (threadIdx.x == 32 && atomicAdd(&a.status->finished, 1u) == gridDim.x - 1) {
-        __threadfence();
-        a.status->last = atomicExch(&a.status->current, (int32_t)WINO_OK);
     }
     if (a.tokens)
-        eq4_tail(a, row0, per_seq, status, s_done, s_ndone, sm);
+        eq4_tail(a, row0, status, s_done, s_ndone, sm);
+    publish_status(a, status, a.tokens ? a.N / a.seq_rows : 0);
 }
 
 // Eq. 4 alone, one CTA per sequence.
@@ -354,7 +500,11 @@ __global__ void __launch_bounds__(kFinishRows * 32)
                         const wino_params p, int32_t *counts, int8_t *flags)
 {
     __shared__ Eq4Smem sm;
-    eq4_block(blockIdx.x, blockIdx.x, tokens, argmax, pmax, ptarget, p, counts, flags, WINO_OK, sm);
+    const int s = blockIdx.x;
+    const int64_t rows = ((p.options & (WINO_OPT_NO_SHADOW | WINO_OPT_COMPACT)) ? 1 : 2) * (int64_t)p.blk_len;
+    int32_t yv[kEq4Per];
+    load_tokens(tokens, s, p, yv);
+    eq4_block<false>(s, yv, seq_stats(argmax, pmax, ptarget, s * rows, p), tokens, p, counts, flags, WINO_OK, sm);
 }
 
 // Row compaction: one CTA per position copies the one row Eq. 4 will read -- the block row of a masked
@@ -446,19 +596,28 @@ cudaError_t launch_gather_active(const uint16_t *H, uint16_t *Hc, int32_t *targe
                               reinterpret_cast<uint4 *>(Hc), target, tokens, p, d / 8);
 }
 
-cudaError_t launch_finish(const FinishArgs &a, cudaStream_t stream)
+cudaError_t launch_finish(FinishArgs a, cudaStream_t stream)
 {
+    const wino_params &p = a.p;
+    a.seq_rows = a.tokens ? ((p.options & (WINO_OPT_NO_SHADOW | WINO_OPT_COMPACT)) ? 1 : 2) * p.blk_len : 0;
+    const bool clusters = a.tokens && a.seq_rows <= kClusterSeqRows;
+    a.cluster = clusters ? std::min(8, (a.seq_rows + kFinishRows - 1) / kFinishRows) : 1;  // 8: the portable most
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((a.N + kFinishRows - 1) / kFinishRows));
+    cfg.gridDim = dim3(clusters ? (unsigned)(a.N / a.seq_rows * a.cluster)
+                                : (unsigned)((a.N + kFinishRows - 1) / kFinishRows));
     cfg.blockDim = dim3(kFinishRows * 32);
-    cfg.dynamicSmemBytes = a.tokens ? conf_bytes(a.p) : 0;
+    cfg.dynamicSmemBytes = (a.tokens ? conf_bytes(p) : 0) + (clusters ? 12u * (uint32_t)a.seq_rows : 0);
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)a.cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, finish_kernel, a);
+    cfg.numAttrs = clusters ? 2 : 1;
+    return clusters ? cudaLaunchKernelEx(&cfg, finish_step_kernel, a) : cudaLaunchKernelEx(&cfg, finish_kernel, a);
 }
 
 cudaError_t launch_draft_verify(int32_t *tokens, const int32_t *argmax, const float *pmax, const float *ptarget,

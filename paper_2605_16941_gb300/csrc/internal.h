@@ -104,10 +104,10 @@ constexpr int kMaxRecordsPerRow = 256;
 // Status words at the start of every workspace.  `current` collects the
 // errors of the call in flight: score-kernel CTAs record theirs only after
 // griddepcontrol.wait (so after the previous call's finish kernel has cleared
-// the word), and the finish kernel adds its own.  The last finish CTA of a call
-// publishes `current` as `last` (what wino_read_device_status returns) and
-// clears it for the next call; `finished` counts the finish CTAs done with the
-// call and is reset by the next call's score kernel.  A workspace starts zeroed.
+// the word).  The finish kernel publishes the outcome as `last` (what
+// wino_read_device_status returns); only after a failure does it clear
+// `current` for the next call, by the last of its CTAs, which `finished` counts
+// (zero between calls).  A workspace starts zeroed.
 struct StatusWords {
     int32_t current;
     int32_t last;
@@ -145,7 +145,7 @@ struct FinishArgs {
     float *entropy;       // optional: H(p) = -sum_v p_v log p_v per row
     int32_t G, N, V;      // G: records per row
     TargetSource ts;
-    StatusWords *status;  // read; WINO_ERR_ARG added when an active-sequence list entry is out of range
+    StatusWords *status;  // read and published; WINO_ERR_ARG when an active-sequence list entry is out of range
     int32_t *argmax;
     float *pmax;
     float *ptarget;
@@ -155,6 +155,9 @@ struct FinishArgs {
     int32_t *counts;
     int8_t *flags;
     int32_t *tickets;  // [n_seq], zero on entry
+    // set by launch_finish
+    int32_t seq_rows;  // rows of a sequence
+    int32_t cluster;   // CTAs per sequence (finish_step_kernel)
 };
 
 // Work split of one score launch: tile width bn, number of row-block groups and pairs per group, for
@@ -200,7 +203,7 @@ cudaError_t launch_score_vmajor(const CUtensorMap &tmH, const CUtensorMap &tmW, 
 cudaLaunchConfig_t score_launch_config(unsigned grid, unsigned threads, uint32_t smem, cudaStream_t stream,
                                        cudaLaunchAttribute (&attr)[2]);
 
-cudaError_t launch_finish(const FinishArgs &a, cudaStream_t stream);
+cudaError_t launch_finish(FinishArgs a, cudaStream_t stream);
 
 // Row compaction (WINO_OPT_COMPACT): Hc[s*L + l] = H[(2s + (tokens[s, b0 + l] == MASK ? 0 : 1)) * L + l].
 cudaError_t launch_gather_active(const uint16_t *H, uint16_t *Hc, int32_t *target, const int32_t *tokens,

@@ -168,8 +168,6 @@ __global__ void __launch_bounds__(kVmThreads, 1)
 
     if (warp >= 2 || !tmem_ok) {
         ptx::grid_dep_wait();
-        if (blockIdx.x == 0 && threadIdx.x == 64)
-            a.status->finished = 0;  // the previous call's finish kernel has completed
         if (tl && threadIdx.x == 64)
             tl[3] = ptx::globaltimer_ns();
         if (threadIdx.x >= 64)
