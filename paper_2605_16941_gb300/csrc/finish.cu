@@ -10,7 +10,7 @@
 //   H(p)     = -sum_v p_v log p_v = ln Z - sum_v exp(l_v - m) (l_v - m) / Z
 // that WINO+'s deferral and sharpening terms use (Sec. 5.3, Eq. 6-7).  In a whole step (wino_step) Eq. 4 follows in
 // the same launch:
-//   finish_step_kernel, sequences of up to 128 rows: a cluster of CTAs per sequence merges its rows and hands the
+//   finish_step_kernel, sequences of up to 256 rows: a cluster of CTAs per sequence merges its rows and hands the
 //     statistics to its first CTA, which applies Eq. 4;
 //   finish_kernel, longer sequences: every CTA adds its merged rows to its sequences' tickets (cleared by the score
 //     kernel of the same step), and the CTA that completes a sequence applies Eq. 4.
@@ -44,23 +44,21 @@ namespace wino {
 namespace {
 
 constexpr float kLn2 = 0.6931471805599453f;
-constexpr int kFinishRows = 8;  // rows (warps) per finish CTA; also the CTA size of the Eq. 4 kernels
-constexpr int kClusterSeqRows = 128;  // rows of a sequence up to which a cluster of CTAs finishes it: two rows per warp
+constexpr int kFinishRows = 8;  // rows (warps) per finish_kernel CTA; also the CTA size of draft_verify_kernel
+constexpr int kClusterSeqRows = 256;  // rows of a sequence up to which a cluster of CTAs finishes it: two per warp
 constexpr int kRecInFlight = 5;  // records each lane loads at once (160 per row: two per pair of a 76-pair launch fit)
 
 // Block-wide reduction scratch for eq4_block.
+template <int kWarps>
 struct Eq4Smem {
-    int32_t i0[kFinishRows], i1[kFinishRows], i2[kFinishRows];
-    float f0[kFinishRows];
+    int32_t i0[kWarps], i1[kWarps], i2[kWarps];
+    float f0[kWarps];
 };
 
 // Dynamic shared memory of a launch with fixed-M drafting: pmax of each masked position, -inf elsewhere.  (Static, it
 // would keep the CTA from fitting beside a score CTA, see kScoreSmemMax.)
 extern __shared__ float s_conf[];
 inline uint32_t conf_bytes(const wino_params &p) { return p.draft_m > 0 ? (uint32_t)p.blk_len * 4u : 0u; }
-
-constexpr int kEq4Threads = kFinishRows * 32;
-constexpr int kEq4Per = kMaxBlkLen / kEq4Threads;  // positions per thread
 
 // Where Eq. 4 finds a sequence's statistics: entry l of argmax and pmax belongs to the row read for a masked position
 // l, entry l of ptarget to the row read for a decoded one.
@@ -77,26 +75,28 @@ __device__ __forceinline__ SeqStats seq_stats(const int32_t *argmax, const float
     return SeqStats{argmax + first, pmax + first, ptarget ? ptarget + first + (both ? p.blk_len : 0) : nullptr};
 }
 
-// The current tokens of sequence s's block, thread t's positions t, t + 256, ...
-__device__ __forceinline__ void load_tokens(const int32_t *tokens, int s, const wino_params &p, int32_t (&yv)[kEq4Per])
+// The current tokens of sequence s's block, thread t's positions t, t + 32 * kWarps, ...
+template <int kWarps>
+__device__ __forceinline__ void load_tokens(const int32_t *tokens, int s, const wino_params &p,
+                                            int32_t (&yv)[kMaxBlkLen / (32 * kWarps)])
 {
     const int32_t *y = tokens + (int64_t)s * p.seq_len + p.blk_start;
 #pragma unroll
-    for (int i = 0; i < kEq4Per; ++i) {
-        const int l = (int)threadIdx.x + i * kEq4Threads;
+    for (int i = 0; i < kMaxBlkLen / (32 * kWarps); ++i) {
+        const int l = (int)threadIdx.x + i * 32 * kWarps;
         yv[i] = l < p.blk_len ? y[l] : 0;
     }
 }
 
-// Eq. 4 on sequence s, whose block holds the tokens yv, by the whole CTA.  Every load is issued before any decision so
+// Eq. 4 on sequence s, whose block holds the tokens yv, by the whole CTA of kWarps warps.  Every load is issued before any decision so
 // the update costs about one memory round trip.  kShared: the statistics are in this CTA's shared memory; otherwise
 // they are read through L2, as other CTAs of the same launch may have written them.
-template <bool kShared>
-__device__ void eq4_block(int s, const int32_t (&yv)[kEq4Per], const SeqStats st, int32_t *tokens, const wino_params &p,
-                          int32_t *counts, int8_t *flags, int32_t status, Eq4Smem &sm)
+template <bool kShared, int kWarps>
+__device__ void eq4_block(int s, const int32_t (&yv)[kMaxBlkLen / (32 * kWarps)], const SeqStats st, int32_t *tokens,
+                          const wino_params &p, int32_t *counts, int8_t *flags, int32_t status, Eq4Smem<kWarps> &sm)
 {
-    constexpr int kT = kEq4Threads;
-    constexpr int kPer = kEq4Per;
+    constexpr int kT = 32 * kWarps;
+    constexpr int kPer = kMaxBlkLen / kT;  // positions per thread
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (status != WINO_OK) {  // the scores of this step are invalid: leave the state alone
         if (tid < 3)
@@ -158,7 +158,7 @@ __device__ void eq4_block(int s, const int32_t (&yv)[kEq4Per], const SeqStats st
     best = -INFINITY;
     best_l = INT32_MAX;
 #pragma unroll
-    for (int w = 0; w < kFinishRows; ++w) {
+    for (int w = 0; w < kWarps; ++w) {
         n_clear += sm.i0[w];
         n_mask += sm.i1[w];
         if (sm.f0[w] > best || (sm.f0[w] == best && sm.i2[w] < best_l)) {
@@ -249,7 +249,7 @@ __device__ void eq4_block(int s, const int32_t (&yv)[kEq4Per], const SeqStats st
         const int32_t *src = tid == 0 ? sm.i0 : (tid == 1 ? sm.i1 : sm.i2);
         int32_t v = 0;
 #pragma unroll
-        for (int w = 0; w < kFinishRows; ++w)
+        for (int w = 0; w < kWarps; ++w)
             v += src[w];
         counts[s * 3 + tid] = v;
     }
@@ -369,12 +369,14 @@ __device__ __forceinline__ void publish_status(const FinishArgs &a, int32_t stat
 // 4.3 KB of shared memory they started only when score CTAs left: 9.5 -> 8.5 us for the tiny step in a CUDA graph).
 // Handing over through global memory (finish_kernel: one CTA per 8 rows, fences, a ticket per sequence, the statistics
 // read back) costs about 3 us more, but merges more rows at once.  us per step, finish_kernel -> here: 64 rows 9.2 ->
-// 7.9 (d = 64, V = 1000), 151.0 -> 147.8 (d = 4096, V = 126464); 128 rows 9.3 -> 8.5; 256 rows 12.2 -> 13.0 and 512 rows
-// 10.3 -> 13.4, so longer sequences stay with finish_kernel.
-__global__ void __launch_bounds__(kFinishRows * 32, 5) finish_step_kernel(const FinishArgs a)
+// 7.9 (d = 64, V = 1000), 151.0 -> 147.8 (d = 4096, V = 126464); 128 rows 9.3 -> 8.5.  Above 128 rows with 16 warps per
+// CTA instead of 8: 192 rows 12.3 -> 11.6, 256 rows 11.9 -> 11.5 (d = 256, V = 20000; with 8 warps 13.0).  512 rows took
+// 13.4 against 10.3, so longer sequences stay with finish_kernel.
+template <int kWarps>
+__global__ void __maxnreg__(48) finish_step_kernel(const FinishArgs a)
 {
     ptx::grid_dep_launch_dependents();  // the next call may start streaming its H and W
-    __shared__ Eq4Smem sm;
+    __shared__ Eq4Smem<kWarps> sm;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = ptx::cluster_ctarank();
     const int seq = (int)blockIdx.x / a.cluster, R = a.seq_rows;
@@ -384,14 +386,14 @@ __global__ void __launch_bounds__(kFinishRows * 32, 5) finish_step_kernel(const 
     ptx::cluster_sync();  // the first CTA has started: its shared memory may be written
     ptx::grid_dep_wait();
     const int32_t status = *reinterpret_cast<const volatile int32_t *>(&a.status->current);
-    int32_t yv[kEq4Per];
+    int32_t yv[kMaxBlkLen / (32 * kWarps)];
     int s = -1;
     if (rank == 0 && !bad_entry(a.p, seq)) {
         s = a.p.active_seq ? a.p.active_seq[seq] : seq;
-        load_tokens(a.tokens, s, a.p, yv);
+        load_tokens<kWarps>(a.tokens, s, a.p, yv);
     }
     const int64_t first = (int64_t)seq * R;
-    const int stride = a.cluster * kFinishRows;
+    const int stride = a.cluster * kWarps;
     auto hand_over = [&](int r, const Merged &o) {  // row r of the sequence, by lane 0
         const RowStats x = row_stats(o, status);
         store_row(a, first + r, x);
@@ -399,7 +401,7 @@ __global__ void __launch_bounds__(kFinishRows * 32, 5) finish_step_kernel(const 
         ptx::st_shared_cluster_u32(ptx::mapa(ptx::smem_u32(s_pmax + r), 0), __float_as_uint(x.pmax));
         ptx::st_shared_cluster_u32(ptx::mapa(ptx::smem_u32(s_ptarget + r), 0), __float_as_uint(x.ptarget));
     };
-    int r = (int)rank * kFinishRows + warp;
+    int r = (int)rank * kWarps + warp;
     if (R <= stride) {  // one row per warp
         if (r < R) {
             Merged o[1];
@@ -422,14 +424,14 @@ __global__ void __launch_bounds__(kFinishRows * 32, 5) finish_step_kernel(const 
     __syncwarp();
     ptx::cluster_sync();  // the statistics are in the first CTA's shared memory
     if (s >= 0)
-        eq4_block<true>(s, yv, seq_stats(s_argmax, s_pmax, s_ptarget, 0, a.p), a.tokens, a.p, a.counts, a.flags, status,
+        eq4_block<true, kWarps>(s, yv, seq_stats(s_argmax, s_pmax, s_ptarget, 0, a.p), a.tokens, a.p, a.counts, a.flags, status,
                         sm);
     publish_status(a, status, a.N / R);
 }
 
 // Eq. 4 at the end of finish_kernel: the CTA that merges the last rows of a sequence updates that sequence.
 __device__ void eq4_tail(const FinishArgs &a, int64_t row0, int32_t status, int32_t *s_done, int32_t &s_ndone,
-                         Eq4Smem &sm)
+                         Eq4Smem<kFinishRows> &sm)
 {
     __syncthreads();
     const int64_t per_seq = a.seq_rows;
@@ -454,9 +456,9 @@ __device__ void eq4_tail(const FinishArgs &a, int64_t row0, int32_t status, int3
         if (bad_entry(a.p, sq))
             continue;  // no update (the status says so)
         const int s = a.p.active_seq ? a.p.active_seq[sq] : sq;
-        int32_t yv[kEq4Per];
-        load_tokens(a.tokens, s, a.p, yv);
-        eq4_block<false>(s, yv, seq_stats(a.argmax, a.pmax, a.ptarget, sq * per_seq, a.p), a.tokens, a.p, a.counts,
+        int32_t yv[kMaxBlkLen / (32 * kFinishRows)];
+        load_tokens<kFinishRows>(a.tokens, s, a.p, yv);
+        eq4_block<false, kFinishRows>(s, yv, seq_stats(a.argmax, a.pmax, a.ptarget, sq * per_seq, a.p), a.tokens, a.p, a.counts,
                          a.flags, status, sm);
     }
 }
@@ -469,7 +471,7 @@ __global__ void __launch_bounds__(kFinishRows * 32, 5) finish_kernel(const Finis
     ptx::grid_dep_launch_dependents();  // the next call may start streaming its H and W
     __shared__ int32_t s_done[kFinishRows];
     __shared__ int32_t s_ndone;
-    __shared__ Eq4Smem sm;
+    __shared__ Eq4Smem<kFinishRows> sm;
     const int64_t row0 = (int64_t)blockIdx.x * kFinishRows;
     const int64_t row = row0 + (threadIdx.x >> 5);
     ptx::grid_dep_wait();
@@ -499,12 +501,12 @@ __global__ void __launch_bounds__(kFinishRows * 32)
     draft_verify_kernel(int32_t *tokens, const int32_t *argmax, const float *pmax, const float *ptarget,
                         const wino_params p, int32_t *counts, int8_t *flags)
 {
-    __shared__ Eq4Smem sm;
+    __shared__ Eq4Smem<kFinishRows> sm;
     const int s = blockIdx.x;
     const int64_t rows = ((p.options & (WINO_OPT_NO_SHADOW | WINO_OPT_COMPACT)) ? 1 : 2) * (int64_t)p.blk_len;
-    int32_t yv[kEq4Per];
-    load_tokens(tokens, s, p, yv);
-    eq4_block<false>(s, yv, seq_stats(argmax, pmax, ptarget, s * rows, p), tokens, p, counts, flags, WINO_OK, sm);
+    int32_t yv[kMaxBlkLen / (32 * kFinishRows)];
+    load_tokens<kFinishRows>(tokens, s, p, yv);
+    eq4_block<false, kFinishRows>(s, yv, seq_stats(argmax, pmax, ptarget, s * rows, p), tokens, p, counts, flags, WINO_OK, sm);
 }
 
 // Row compaction: one CTA per position copies the one row Eq. 4 will read -- the block row of a masked
@@ -601,11 +603,12 @@ cudaError_t launch_finish(FinishArgs a, cudaStream_t stream)
     const wino_params &p = a.p;
     a.seq_rows = a.tokens ? ((p.options & (WINO_OPT_NO_SHADOW | WINO_OPT_COMPACT)) ? 1 : 2) * p.blk_len : 0;
     const bool clusters = a.tokens && a.seq_rows <= kClusterSeqRows;
-    a.cluster = clusters ? std::min(8, (a.seq_rows + kFinishRows - 1) / kFinishRows) : 1;  // 8: the portable most
+    const int warps = clusters && a.seq_rows > 128 ? 16 : kFinishRows;
+    a.cluster = clusters ? std::min(8, (a.seq_rows + warps - 1) / warps) : 1;  // 8: the portable most
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(clusters ? (unsigned)(a.N / a.seq_rows * a.cluster)
                                 : (unsigned)((a.N + kFinishRows - 1) / kFinishRows));
-    cfg.blockDim = dim3(kFinishRows * 32);
+    cfg.blockDim = dim3((unsigned)warps * 32);
     cfg.dynamicSmemBytes = (a.tokens ? conf_bytes(p) : 0) + (clusters ? 12u * (uint32_t)a.seq_rows : 0);
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
@@ -617,7 +620,10 @@ cudaError_t launch_finish(FinishArgs a, cudaStream_t stream)
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = clusters ? 2 : 1;
-    return clusters ? cudaLaunchKernelEx(&cfg, finish_step_kernel, a) : cudaLaunchKernelEx(&cfg, finish_kernel, a);
+    if (!clusters)
+        return cudaLaunchKernelEx(&cfg, finish_kernel, a);
+    return warps == 16 ? cudaLaunchKernelEx(&cfg, finish_step_kernel<16>, a)
+                       : cudaLaunchKernelEx(&cfg, finish_step_kernel<8>, a);
 }
 
 cudaError_t launch_draft_verify(int32_t *tokens, const int32_t *argmax, const float *pmax, const float *ptarget,

@@ -1,4 +1,4 @@
-"""The end of a step on both sides of the row count up to which a cluster of CTAs finishes a sequence (128 rows), down
+"""The end of a step on both sides of the row count up to which a cluster of CTAs finishes a sequence (256 rows), down
 to one row: wino_step leaves exactly the tokens, counts, flags and finalization steps that wino_score_rows with the
 same targets followed by wino_draft_verify (its statistics read from global memory, one CTA per sequence) gives."""
 import numpy as np
@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("draft_m", [0, 3])
 @pytest.mark.parametrize("no_shadow", [False, True], ids=["verify", "no_shadow"])
-@pytest.mark.parametrize("L", [1, 4, 5, 33, 63, 64, 65, 128, 129])
+@pytest.mark.parametrize("L", [1, 4, 5, 33, 63, 64, 65, 128, 129, 256, 257])
 def test_step_equals_score_then_draft_verify(L, no_shadow, draft_m):
     import paper_2605_16941_gb300 as wino
     from gpu_helpers import dev
