@@ -128,7 +128,8 @@ struct ScoreArgs {
     int32_t stages;            // ring stages, 2..kMaxStages
     uint32_t stage_bytes;      // 16 KB + stage_bytes_w(bn) + a pass's third slot (W, or 16 KB of H)
     int32_t n_groups, G;
-    int32_t hw[2], slots;  // vocabulary-major kernel only: rows of each accumulator of a tile, accumulators in TMEM
+    int32_t hw[2], slots;  // vocabulary-major kernel only: rows of each accumulator of a tile, accumulators in TMEM,
+    int32_t split;         // 1: the last round's tiles are shared by two pairs, one accumulator each
     TargetSource ts;
     float4 *part;       // [N][records per row: G, or 2 G (one per CTA) from the vocabulary-major kernel]
     float *part_u;      // the same shape, entropy variant only: sum of exp(l - m) * (l - m) * log2(e) over the pair's tiles
@@ -174,7 +175,7 @@ ScoreSchedule score_schedule(int32_t n_mb, int64_t V, int max_units, int32_t rec
 // the launch (its rule stands in score_vmajor.cu); `rows` is the split score.cu would use.
 struct VmSchedule {
     int32_t bn, n_vt, n_groups, G;
-    int32_t hw[2], slots, stages;
+    int32_t hw[2], slots, split, stages;
     uint32_t stage_bytes;
     int64_t cost;  // estimated ns
 };

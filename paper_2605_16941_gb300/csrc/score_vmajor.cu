@@ -45,8 +45,8 @@ constexpr int kMaxChunks = 4;  // 32-column chunks of one accumulator (256 colum
 // and 700 for its epilogue, or the epilogue alone (9.7 ns a column) if that is longer, and the last tile's epilogue.
 // On 70 random shapes (N to 2048, d to 4096, V from 19456) the choice was within 4 % of the best split of either kernel
 // on 65, and at worst 12 % off it and 7 % slower than score.cu.
-// us per step, score.cu -> here (groups), d = 4096, V = 126464: N = 288 308 -> 220 (1), 320 316 -> 243 (1),
-// 384 326 -> 287 (1, 2), 448 333 -> 312 (2), 512 344 -> 346 (2), 576 494 -> 390 (2), 640 502 -> 421 (2),
+// us per step, score.cu -> here (groups), d = 4096, V = 126464: N = 288 308 -> 216 (1), 320 316 -> 243 (1),
+// 384 326 -> 271 (1), 448 333 -> 312 (2), 512 344 -> 346 (2), 576 494 -> 390 (2), 640 502 -> 421 (2),
 // 768 523 -> 482 (3), 896 616 -> 578 (4), 1024 632 -> 620 (4), 1280 870 -> 771 (5), 1664 1171 -> 1036 (4), 2048
 // 1204 -> 1213 (stays with score.cu); d = 1024, V = 64000: 300 52.8 -> 41.5 (2), 448 54.4 -> 50.3 (2), 512 55.4 -> 54.8
 // (2); d = 512, V = 32000: 384 24.0 -> 23.2 (2), 448 24.1 -> 24.5 (stays); d = 256, V = 64000: 384 26.0 -> 29.3 (stays).
@@ -74,6 +74,23 @@ struct alignas(8) VmBarriers {
     int32_t abort;
 };
 static_assert(sizeof(VmBarriers) <= kVmBarrierBytes, "barrier block must fit its reserve");
+
+// Item i of the pair at column `col` of its group: vocabulary tile vt, accumulators [h0, h1).  Rounds of whole tiles
+// col, col + G, ...; in a last round that would leave at least half of the pairs idle (ScoreArgs::split), a tile's two
+// accumulators go to two pairs (V = 126464 on 76 pairs: 6.5 tiles a pair instead of 7; us per step at d = 4096, N = 288
+// 215.5 -> 209.5, 300 222.5 -> 217.5, 384 275.3 -> 270.3, steady state; 352 at full clock 229 -> 219).
+struct VmItem {
+    int vt, h0, h1;
+};
+__device__ __forceinline__ bool vm_item(const ScoreArgs &a, int col, int i, VmItem &it)
+{
+    const int full = a.n_vt / a.G, rem = a.n_vt - full * a.G;
+    const bool half = a.split && i == full;
+    it.vt = i * a.G + (half ? col >> 1 : col);
+    it.h0 = half ? col & 1 : 0;
+    it.h1 = half ? it.h0 + 1 : (a.hw[1] > 0 ? 2 : 1);
+    return half ? col < 2 * rem : it.vt < a.n_vt;
+}
 
 // Running state of one row in one thread (the four partial sums of a fold are added up after each fold).
 struct ColState {
@@ -119,7 +136,6 @@ __global__ void __launch_bounds__(kVmThreads, 1)
 
     const int S = a.stages;
     const int hw0 = a.hw[0], hw1 = a.hw[1], slots = a.slots;  // hw1 = 0: one accumulator per tile
-    const int halves = hw1 > 0 ? 2 : 1;
     const int hrows = (hw0 + hw1) >> 1;  // rows of H this CTA stages per K slice
     const int half_bn = a.bn >> 1;      // vocabulary rows this CTA stages per tile
     auto sA = [&](int s) { return ring + (uint32_t)s * a.stage_bytes; };
@@ -192,7 +208,8 @@ __global__ void __launch_bounds__(kVmThreads, 1)
             uint32_t phase = 0;
             int64_t issued = 0;
             bool aborted = false;
-            for (int vt = col; vt < a.n_vt && !aborted; vt += a.G) {
+            VmItem it;
+            for (int i = 0; !aborted && vm_item(a, col, i, it); ++i) {
                 for (int kb = 0; kb < a.n_kb; ++kb) {
                     if (!wait_bounded(empty(stage), phase ^ 1u, &bars->abort)) {
                         aborted = true;
@@ -201,7 +218,7 @@ __global__ void __launch_bounds__(kVmThreads, 1)
                     const uint32_t bar = ptx::mapa(full(stage), 0);  // the leader's stage barrier
                     if (leader)
                         ptx::mbar_arrive_expect_tx(full(stage), stage_tx);
-                    ptx::tma_load_2d_pair(sA(stage), &tmW, bar, w_x(kb), w_y(kb, vt * a.bn + (int)rank * half_bn),
+                    ptx::tma_load_2d_pair(sA(stage), &tmW, bar, w_x(kb), w_y(kb, it.vt * a.bn + (int)rank * half_bn),
                                           pol_w);
                     ptx::tma_load_2d_pair(sB(stage, 0), &tmH, bar, kb * kBK, row0 + (int)rank * hrows, pol_h);
                     if (tl && issued == 0)
@@ -241,16 +258,18 @@ __global__ void __launch_bounds__(kVmThreads, 1)
                 for (int k = 0; k < kBK / 16; ++k)  // +32 B along K per MMA = +2 in the encoded address
                     ptx::mma_bf16_pair(dst, da + 2u * k, db + 2u * k, idesc, (kb | k) != 0);
             };
-            for (int vt = col; vt < a.n_vt && !aborted; vt += a.G) {
+            VmItem it;
+            for (int i = 0; !aborted && vm_item(a, col, i, it); ++i) {
+                const bool both = it.h1 - it.h0 == 2;
                 const int acc0 = slot;
                 const uint32_t par0 = (round & 1u) ^ 1u;
                 if (++slot == slots) {
                     slot = 0;
                     ++round;
                 }
-                const int acc1 = slot;  // with two accumulators per tile
+                const int acc1 = slot;  // with both accumulators of a tile
                 const uint32_t par1 = (round & 1u) ^ 1u;
-                if (halves == 2 && ++slot == slots) {
+                if (both && ++slot == slots) {
                     slot = 0;
                     ++round;
                 }
@@ -260,7 +279,7 @@ __global__ void __launch_bounds__(kVmThreads, 1)
                     break;
                 }
                 ptx::tc_fence_after();
-                bool second = halves == 1;  // the second accumulator is free (or not used)
+                bool second = !both;        // the second accumulator is free (or not used)
                 int held = 0;               // K slices whose second-accumulator MMAs have not been issued: [0, held)
                 const int s0 = stage;
                 for (int kb = 0; kb < a.n_kb; ++kb) {
@@ -268,11 +287,11 @@ __global__ void __launch_bounds__(kVmThreads, 1)
                         aborted = true;
                         break;
                     }
-                    issue(acc0, stage, 0, kb);
+                    issue(acc0, stage, it.h0, kb);
                     if (kb == a.n_kb - 1)  // accumulator 0 is done: its epilogue need not wait for accumulator 1
                         ptx::mma_commit_pair_multicast(tfull(acc0), kBothCtas);
                     if (second) {
-                        if (halves == 2)
+                        if (both)
                             issue(acc1, stage, 1, kb);
                         ptx::mma_commit_pair_multicast(empty(stage), kBothCtas);
                     } else {
@@ -304,9 +323,9 @@ __global__ void __launch_bounds__(kVmThreads, 1)
                 }
                 if (aborted)
                     break;
-                if (halves == 2)
+                if (both)
                     ptx::mma_commit_pair_multicast(tfull(acc1), kBothCtas);
-                ++tiles;
+                tiles += it.h0 == 0;
             }
             // No MMA may still be writing either CTA's TMEM when it is released.
             ptx::mma_commit_pair(mma_done);
@@ -344,12 +363,13 @@ __global__ void __launch_bounds__(kVmThreads, 1)
         }
         int use = 0;
         bool aborted = false;
-        for (int vt = col; vt < a.n_vt && !aborted; vt += a.G) {
-            const int v0 = vt * a.bn + (int)rank * half_bn + q * 32;  // vocabulary id of this warp's first lane
+        VmItem it;
+        for (int i = 0; !aborted && vm_item(a, col, i, it); ++i) {
+            const int v0 = it.vt * a.bn + (int)rank * half_bn + q * 32;  // vocabulary id of this warp's first lane
             const int nvalid = min(half_bn - q * 32, a.V - v0);       // valid lanes from there (may be <= 0)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                if (h >= halves || aborted)
+                if (h < it.h0 || h >= it.h1 || aborted)
                     continue;
                 const int slot = use % slots;
                 int ok = 1;
@@ -363,12 +383,12 @@ __global__ void __launch_bounds__(kVmThreads, 1)
                 }
                 if (nvalid > 0) {
 #pragma unroll
-                    for (int i = 0; i < kMaxChunks; ++i) {
-                        const int k = h * kMaxChunks + i;
+                    for (int c = 0; c < kMaxChunks; ++c) {
+                        const int k = h * kMaxChunks + c;
                         if (!(live >> k & 1u))
                             continue;
                         float x[32];
-                        ptx::tmem_ld_32x32b_x32(lanes + (uint32_t)(slot * hw0 + chunk_of(h, i) * 32), x);
+                        ptx::tmem_ld_32x32b_x32(lanes + (uint32_t)(slot * hw0 + chunk_of(h, c) * 32), x);
                         ptx::tmem_ld_wait();
                         // transpose: row j (of the chunk), vocabulary lane l at j * 32 + ((l / 4) ^ (j % 8)) * 4 + l % 4
 #pragma unroll
@@ -499,7 +519,9 @@ bool vm_split(int64_t N, int64_t n_kb, int64_t V, int max_units, int32_t records
     const int64_t w = s.hw[0] + s.hw[1], chunks = (s.hw[0] + 31) / 32 + (s.hw[1] + 31) / 32;
     const int64_t mma = s.hw[1] > 0 ? n_kb * (60 + w * 7 / 5) + 4 * w : n_kb * (190 + w * 3 / 4);
     const int64_t epilogue = (chunks + 1) / 2 * 992;
-    s.cost = epilogue + tiles * (mma > epilogue ? mma : epilogue);
+    const int64_t tile = mma > epilogue ? mma : epilogue, rem = s.n_vt % s.G;
+    s.split = s.hw[1] > 0 && rem > 0 && 2 * rem <= s.G;
+    s.cost = epilogue + tiles * tile - (s.split ? tile * 3 / 10 : 0);
     s.stage_bytes = kVmStageBytesW + (uint32_t)((s.hw[0] + s.hw[1]) / 2) * 128u;
     const uint32_t fit = kVmRingCapacity / s.stage_bytes;
     s.stages = (int32_t)(fit < (uint32_t)kVmMaxStages ? fit : (uint32_t)kVmMaxStages);

@@ -269,6 +269,7 @@ int score_and_finish(const uint16_t *H, const uint16_t *W, bool w_panels, int64_
     a.hw[0] = vm.hw[0];
     a.hw[1] = vm.hw[1];
     a.slots = vm.slots;
+    a.split = vm.split;
     a.ts = ts;
     a.part = reinterpret_cast<float4 *>(w8 + L.part);
     a.part_u = entropy ? reinterpret_cast<float *>(w8 + L.part_u) : nullptr;

@@ -25,6 +25,8 @@ SHAPES = [
     (390, 1024, 24118, 2 * 95),    # 208 columns
     (530, 1024, 25672, 2 * 101),   # two groups of 144 + 128 columns, the second ragged
     (726, 1024, 24118, 3 * 95),    # 256 columns
+    (257, 2056, 19457, 1 * 77),    # a last tile of one entry whose two accumulators go to two pairs, K tail
+    (581, 512, 42766, 2 * 168),    # two groups, 16 last tiles shared by 32 of each group's 38 pairs
 ]
 
 
