@@ -131,10 +131,12 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// Arrive on an mbarrier of any CTA of the cluster (release at cluster scope).
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
+// Arrive on an mbarrier of any CTA of the cluster, without ordering this thread's earlier memory accesses: for signals
+// that publish no memory writes, such as "accumulator read" (tensor-memory loads complete at tcgen05.wait::ld and are
+// ordered by the tcgen05 fences on both sides).  A release at cluster scope waits for all of them.
+__device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_addr)
 {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
 // try_wait with acquire at cluster scope: for barriers that other CTAs of the cluster arrive on.

@@ -62,7 +62,10 @@
 //           fold.cuh and accumulator 0 handed over before accumulator 1 is
 //           done (us per step, V = 64000, N = 2048): d = 256 107 -> 74, d = 1024
 //           200 -> 182; d = 4096, V = 126464 1195 -> 1173; three or four warps
-//           per quarter: 72 / 73, 182 / 183, no change.
+//           per quarter: 72 / 73, 182 / 183, no change.  That was with a release
+//           at cluster scope in every accumulator release, a memory barrier that
+//           held each warp for about as long as a chunk's fold; with a relaxed
+//           arrival d = 256 73.4 -> 58.3, d = 1024 168.7 -> 165.5.
 // Work split: see ScoreArgs in internal.h.
 //
 // Every mbarrier wait is bounded (kWaitLimitNs): on expiry the CTA raises an
@@ -382,7 +385,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
             ptx::tc_fence_before();
             __syncwarp();
             if (lane == 0)
-                ptx::mbar_arrive_cluster(ptx::mapa(tempty(i), 0));
+                ptx::mbar_arrive_cluster_relaxed(ptx::mapa(tempty(i), 0));
         };
         auto epilogue_sync = [&] { asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory"); };
         const RowState r0{-INFINITY, 0.f, 0.f, 0.f, 0.f, -INFINITY, 0.f, 0.f, 0.f, 0.f, 0};

@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(kVmThreads, 1)
                 ptx::tc_fence_before();
                 __syncwarp();
                 if (lane == 0)
-                    ptx::mbar_arrive_cluster(ptx::mapa(tempty(slot), 0));
+                    ptx::mbar_arrive_cluster_relaxed(ptx::mapa(tempty(slot), 0));
                 ++use;
             }
         }
