@@ -37,25 +37,27 @@ constexpr int kPrefetchSlices = 4;  // K slices of the first W tile prefetched i
 constexpr int kVmEpiWarps = 8;
 constexpr int kVmThreads = 64 + 32 * kVmEpiWarps;
 constexpr int kMaxChunks = 4;  // 32-column chunks of one accumulator (256 columns) per epilogue warp
-// The split and the choice between the two score kernels: ns on the busiest pair, fitted to steps in steady state
-// (d = 4096, V = 126464, N from 128 to 2048, 1 to 8 groups; d = 256 to 1536 with V from 20000 to 64000; within 5 % of
-// most).  Per tile: n_kb K slices of 190 + 0.75 hw with one accumulator (each SM receives 85 GB/s of W and H), of 60 + 1.4 (hw[0] + hw[1]) with two and 4 ns a
-// column for their epilogue's exposed part, or the epilogue (992 ns for two 32-column chunks, one per warp) if that is
-// longer.  Then the last tile's epilogue.  score.cu: per tile 380 per K slice at bn = 256 (narrower MMAs save less than their columns)
-// and 700 for its epilogue, or the epilogue alone (9.7 ns a column) if that is longer, and the last tile's epilogue.
-// On 70 random shapes (N to 2048, d to 4096, V from 19456) the choice was within 4 % of the best split of either kernel
-// on 65, and at worst 12 % off it and 7 % slower than score.cu.
-// us per step, score.cu -> here (groups), d = 4096, V = 126464: N = 288 308 -> 216 (1), 320 316 -> 243 (1),
-// 384 326 -> 271 (1), 448 333 -> 312 (2), 512 344 -> 346 (2), 576 494 -> 390 (2), 640 502 -> 421 (2),
-// 768 523 -> 482 (3), 896 616 -> 578 (4), 1024 632 -> 620 (4), 1280 870 -> 771 (5), 1664 1171 -> 1036 (4), 2048
-// 1204 -> 1213 (stays with score.cu); d = 1024, V = 64000: 300 52.8 -> 41.5 (2), 448 54.4 -> 50.3 (2), 512 55.4 -> 54.8
-// (2); d = 512, V = 32000: 384 24.0 -> 23.2 (2), 448 24.1 -> 24.5 (stays); d = 256, V = 64000: 384 26.0 -> 29.3 (stays).
+// The split and the choice between the two score kernels: ns on the busiest pair, fitted to calls of both kernels (123
+// and 49 of this one with one and two accumulators per tile, 34 of score.cu, at d = 256 to 2560, rms 5 %, and the d = 4096 rows below).
+// Per tile and K slice, from 24 K slices on (long enough for the board's power limit) and below: one accumulator
+// 190 + 0.75 hw / 204 + 0.22 hw, two 60 + 1.4 (hw[0] + hw[1]) / 1.25 (hw[0] + hw[1]) - 12 and 4 / 8 ns a column once per tile; the
+// epilogue, 540 for two 32-column chunks (one per warp of a quarter), if that is longer, and a third of the shorter of
+// the two on small shapes; then the last tile's epilogue.  score.cu: per tile and K slice 380 (bn + 144) / 400 / 352 (bn - 55) / 201
+// and 700 / 607 once, then its last tile's epilogue.
+// us per step, score.cu -> here (groups), d = 4096, V = 126464: N = 288 308 -> 209 (1), 320 316 -> 238 (1),
+// 384 326 -> 271 (1), 448 333 -> 312 (2), 512 344 -> 346 (2), 576 494 -> 390 (2), 640 502 -> 421 (2), 768 523 -> 482 (3),
+// 896 616 -> 578 (4), 1024 632 -> 620 (4), 1280 870 -> 771 (5), 1664 1171 -> 1036 (4), 2048 1204 -> 1213 (stays with
+// score.cu); d = 1664, V = 64677: 310 71.1 -> 53.0 (1); d = 576, V = 103363: 308 48.6 -> 37.4 (2); d = 512, V = 54379:
+// 1298 67.5 -> 59.9 (6); d = 448, V = 54533: 373 27.1 -> 23.9 (2); d = 512, V = 32000: 448 20.1 (stays); d = 256, V = 64000:
+// 384 19.4 -> 23.9 (2; stays).
+// On the 34 calls the choice was on average within 1 % of the best split of either kernel and at most 1.4 % slower than score.cu.
 // Up to 256 rows (one row block) both kernels follow the W stream.  This one wins where score.cu's mostly
 // empty boxes of H hold it up (N = 32, d = 1024 38.0 -> 30.4; N = 64 30.2 -> 30.9) and where the W stream is long
 // enough for the power limit to bite (d = 3072, V = 126464, N = 128 129 -> 119; d = 4096 168 -> 154, N = 208 175 -> 171,
 // N = 256 183 -> 190; but d = 2048, V = 64000, N = 128 49.6 -> 50.3).
+constexpr int kVmCappedSlices = 24;
 constexpr int kVmShortRows = 48;                        // always here (with a vocabulary for every pair's records)
-constexpr int kVmMinSlices = 4;                         // K slices per tile: below, latencies that the estimates leave out
+constexpr int kVmMinSlices = 5;                         // K slices per tile: below, latencies that the estimates leave out
 constexpr int64_t kVmLongHead = int64_t(1) << 28;       // V * d from which one row block may come here, 512 MiB of W
 constexpr int64_t kRowOneBlockSliceNs = 356;            // a K slice of score.cu's tile of a single row block there
 constexpr int kVmMaxGroups = 8;
@@ -517,10 +519,14 @@ bool vm_split(int64_t N, int64_t n_kb, int64_t V, int max_units, int32_t records
     s.n_vt = (int32_t)((V + bn - 1) / bn);
     s.G = (int32_t)(g < s.n_vt ? g : s.n_vt);
     const int64_t w = s.hw[0] + s.hw[1], chunks = (s.hw[0] + 31) / 32 + (s.hw[1] + 31) / 32;
-    const int64_t mma = s.hw[1] > 0 ? n_kb * (60 + w * 7 / 5) + 4 * w : n_kb * (190 + w * 3 / 4);
-    const int64_t epilogue = (chunks + 1) / 2 * 992;
-    const int64_t tile = mma > epilogue ? mma : epilogue, rem = s.n_vt % s.G;
-    s.split = s.hw[1] > 0 && rem > 0 && 2 * rem <= s.G;
+    const int64_t epilogue = (chunks + 1) / 2 * 540, rem = s.n_vt % s.G;
+    const bool two = s.hw[1] > 0, capped = n_kb >= kVmCappedSlices;
+    const int64_t mma = two ? (capped ? n_kb * (60 + w * 7 / 5) + 4 * w : n_kb * (w * 5 / 4 - 12) + 8 * w)
+                            : n_kb * (capped ? 190 + w * 3 / 4 : 204 + w * 2 / 9);
+    int64_t tile = mma > epilogue ? mma : epilogue;
+    if (!two && !capped)
+        tile += (mma < epilogue ? mma : epilogue) / 3;
+    s.split = two && rem > 0 && 2 * rem <= s.G;
     s.cost = epilogue + tiles * tile - (s.split ? tile * 3 / 10 : 0);
     s.stage_bytes = kVmStageBytesW + (uint32_t)((s.hw[0] + s.hw[1]) / 2) * 128u;
     const uint32_t fit = kVmRingCapacity / s.stage_bytes;
@@ -546,14 +552,15 @@ bool score_vmajor_schedule(int64_t N, int64_t d, int64_t V, int max_units, int32
     }
     if (!found || N <= kVmShortRows)
         return found;
-    const int64_t blocks = (N + kPairM - 1) / kPairM;
-    const int64_t row_tiles = (blocks + rows.n_groups - 1) / rows.n_groups * ((rows.n_vt + rows.G - 1) / rows.G);
     if (n_kb < kVmMinSlices)
         return false;
+    const int64_t blocks = (N + kPairM - 1) / kPairM;
+    const int64_t row_tiles = (blocks + rows.n_groups - 1) / rows.n_groups * ((rows.n_vt + rows.G - 1) / rows.G);
     if (blocks == 1)
         return V * d >= kVmLongHead && out->cost < row_tiles * n_kb * kRowOneBlockSliceNs;
-    const int64_t mma = n_kb * 380 * (rows.bn + 144) / 400 + 700, epilogue = 97 * rows.bn / 10;
-    return out->cost < row_tiles * (mma > epilogue ? mma : epilogue) + epilogue;
+    const int64_t row_tile = n_kb >= kVmCappedSlices ? n_kb * 380 * (rows.bn + 144) / 400 + 700
+                                                     : n_kb * 352 * (rows.bn - 55) / 201 + 607;
+    return out->cost < row_tiles * row_tile + 5 * rows.bn;
 }
 
 cudaError_t launch_score_vmajor(const CUtensorMap &tmH, const CUtensorMap &tmW, const ScoreArgs &a, bool entropy,

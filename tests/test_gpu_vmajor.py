@@ -18,15 +18,15 @@ SHAPES = [
     (1, 8, 19456, 1 * 76),         # one row, one K slice (mostly zero fill), one 32-column chunk
     (33, 72, 20001, 1 * 139),      # 64 columns, K tail, 144-wide tiles, the last one mostly past the vocabulary
     (48, 256, 40000, 1 * 228),     # 176-wide tiles
-    (257, 512, 24118, 3 * 95),     # three groups of one accumulator of 96 columns, the last one ragged
-    (257, 512, 25672, 2 * 101),    # 144 columns: a half chunk at the accumulator's end
-    (257, 512, 38881, 1 * 152),    # 144 + 128 columns, three accumulators in TMEM
-    (327, 1544, 29557, 1 * 116),   # 176 + 160 columns, two accumulators in TMEM
-    (390, 1024, 24118, 2 * 95),    # 208 columns
-    (530, 1024, 25672, 2 * 101),   # two groups of 144 + 128 columns, the second ragged
-    (726, 1024, 24118, 3 * 95),    # 256 columns
-    (257, 2056, 19457, 1 * 77),    # a last tile of one entry whose two accumulators go to two pairs, K tail
-    (581, 512, 42766, 2 * 168),    # two groups, 16 last tiles shared by 32 of each group's 38 pairs
+    (257, 512, 19456, 2 * 76),     # two groups of one accumulator of 144 columns (a half chunk at its end)
+    (392, 512, 19456, 2 * 76),     # 208 columns
+    (482, 512, 19456, 2 * 76),     # 256 columns
+    (257, 1024, 19456, 1 * 76),    # 144 + 128 columns, three accumulators in TMEM
+    (327, 1544, 29557, 1 * 116),   # 176 + 160 columns, two accumulators in TMEM, K and vocabulary tails
+    (518, 1024, 19456, 2 * 76),    # two groups of 144 + 128 columns, the second ragged
+    (257, 2056, 19457, 1 * 77),    # a last tile of one entry whose two accumulators go to two pairs
+    (536, 2048, 20233, 2 * 80),    # two groups, 4 last tiles shared by 8 of each group's 38 pairs
+    (726, 1024, 24118, 3 * 95),    # three groups
 ]
 
 
