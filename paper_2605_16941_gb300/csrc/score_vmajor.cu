@@ -6,9 +6,9 @@
 // vocabulary rows (128 per CTA; bn of them used, as in score.cu's tiles) and N = hw rows of H, a multiple of 16
 // or 32 up to 256, one or two accumulators per vocabulary tile: up to 512 rows of H share each staged W slice, and
 // the padding is at most 31 rows per group.  Up to about 200 rows the MMAs take a fraction of the time of the W
-// stream, which then runs at the copy bandwidth (152.4 us for 1.036 GB at N = 32, 6.8 TB/s; score.cu 157.0 us);
-// from there to 512 rows the shared-memory reads of the MMAs (A is read once per accumulator) and the board's power
-// bound it.
+// stream, which then runs at the copy bandwidth (152.4 us for 1.036 GB at N = 32, 6.8 TB/s; score.cu 157.0 us).
+// From there on the W stream and the MMAs bound it together, and over longer times the board's power (N = 300: W at
+// 80 % of the copy rate with the tensor pipe busy 77 % of the cycles; N = 1024: busy 96 %).
 //
 // The accumulator then has the vocabulary along the TMEM lanes and the rows of H along the columns, so a
 // thread's TMEM load gives 32 different rows' logits of one vocabulary entry.  The epilogue transposes each
@@ -37,20 +37,22 @@ constexpr int kPrefetchSlices = 4;  // K slices of the first W tile prefetched i
 constexpr int kVmEpiWarps = 8;
 constexpr int kVmThreads = 64 + 32 * kVmEpiWarps;
 constexpr int kMaxChunks = 4;  // 32-column chunks of one accumulator (256 columns) per epilogue warp
+
 // The split and the choice between the two score kernels: ns on the busiest pair, fitted to calls of both kernels (123
-// and 49 of this one with one and two accumulators per tile, 34 of score.cu, at d = 256 to 2560, rms 5 %, and the d = 4096 rows below).
-// Per tile and K slice, from 24 K slices on (long enough for the board's power limit) and below: one accumulator
-// 190 + 0.75 hw / 204 + 0.22 hw, two 60 + 1.4 (hw[0] + hw[1]) / 1.25 (hw[0] + hw[1]) - 12 and 4 / 8 ns a column once per tile; the
-// epilogue, 540 for two 32-column chunks (one per warp of a quarter), if that is longer, and a third of the shorter of
-// the two on small shapes; then the last tile's epilogue.  score.cu: per tile and K slice 380 (bn + 144) / 400 / 352 (bn - 55) / 201
-// and 700 / 607 once, then its last tile's epilogue.
+// and 49 of this one with one and two accumulators per tile, 34 of score.cu, at d = 256 to 2560, rms 5 %, and the
+// d = 4096 rows below).  Per tile and K slice, from 24 K slices on (long enough for the board's power limit) and below:
+//   one accumulator    190 + 0.75 hw,                   204 + 0.22 hw;
+//   two                60 + 1.4 w and 4 w per tile,     1.25 w - 12 and 8 w per tile, w = hw[0] + hw[1];
+//   score.cu           0.95 (bn + 144) and 700 per tile, 1.75 (bn - 55) and 607 per tile;
+// here the epilogue (540 for two 32-column chunks, one per warp of a quarter) if that is longer, plus a third of the
+// shorter of the two for one accumulator below 24 K slices; and the last tile's epilogue.
 // us per step, score.cu -> here (groups), d = 4096, V = 126464: N = 288 308 -> 209 (1), 320 316 -> 238 (1),
 // 384 326 -> 271 (1), 448 333 -> 312 (2), 512 344 -> 346 (2), 576 494 -> 390 (2), 640 502 -> 421 (2), 768 523 -> 482 (3),
 // 896 616 -> 578 (4), 1024 632 -> 620 (4), 1280 870 -> 771 (5), 1664 1171 -> 1036 (4), 2048 1204 -> 1213 (stays with
 // score.cu); d = 1664, V = 64677: 310 71.1 -> 53.0 (1); d = 576, V = 103363: 308 48.6 -> 37.4 (2); d = 512, V = 54379:
-// 1298 67.5 -> 59.9 (6); d = 448, V = 54533: 373 27.1 -> 23.9 (2); d = 512, V = 32000: 448 20.1 (stays); d = 256, V = 64000:
-// 384 19.4 -> 23.9 (2; stays).
-// On the 34 calls the choice was on average within 1 % of the best split of either kernel and at most 1.4 % slower than score.cu.
+// 1298 67.5 -> 59.9 (6); d = 448, V = 54533: 373 27.1 -> 23.9 (2); d = 256, V = 64000: 384 19.4 -> 25.6 (3; stays).
+// On those 34 calls the choice was on average within 1 % of the best split of either kernel and at most 1.4 % slower than
+// score.cu; on 36 others that it sent here 7 % faster on average and at most 4 % slower.
 // Up to 256 rows (one row block) both kernels follow the W stream.  This one wins where score.cu's mostly
 // empty boxes of H hold it up (N = 32, d = 1024 38.0 -> 30.4; N = 64 30.2 -> 30.9) and where the W stream is long
 // enough for the power limit to bite (d = 3072, V = 126464, N = 128 129 -> 119; d = 4096 168 -> 154, N = 208 175 -> 171,
