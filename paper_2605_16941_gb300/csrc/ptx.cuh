@@ -82,6 +82,13 @@ __device__ __forceinline__ void cluster_arrive_release()
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
 
+// The same arrival without the release, for barriers that order no memory accesses (a release at cluster scope waits for
+// all of the thread's earlier ones).
+__device__ __forceinline__ void cluster_arrive_relaxed()
+{
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+
 __device__ __forceinline__ void cluster_wait_acquire()
 {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");

@@ -365,9 +365,11 @@ __global__ void __launch_bounds__(kVmThreads, 1)
             if (__any_sync(0xffffffffu, mine))
                 live |= 1u << k;
         }
-        int use = 0;
-        bool aborted = false;
+        int use = 0, n_uses = 0;  // accumulators read, and of all of the pair's items
         VmItem it;
+        for (int i = 0; vm_item(a, col, i, it); ++i)
+            n_uses += it.h1 - it.h0;
+        bool aborted = false;
         for (int i = 0; !aborted && vm_item(a, col, i, it); ++i) {
             const int v0 = it.vt * a.bn + (int)rank * half_bn + q * 32;  // vocabulary id of this warp's first lane
             const int nvalid = min(half_bn - q * 32, a.V - v0);       // valid lanes from there (may be <= 0)
@@ -388,7 +390,10 @@ __global__ void __launch_bounds__(kVmThreads, 1)
                 // Accumulator fully read by this warp: tell the leader's MMA warp.  Sent once the warp's last chunk is in
                 // registers, before its fold: with two accumulators per tile the MMAs wait for it (d = 4096,
                 // V = 126464, N = 352 258.3 -> 255.6 us per step, 600 402 -> 399; with one, no change).
+                // Not sent where the MMA warp does not wait for it (see score.cu's closing barrier).
                 auto release = [&] {
+                    if (use + slots >= n_uses)
+                        return;
                     ptx::tc_fence_before();
                     __syncwarp();
                     if (lane == 0)
@@ -471,7 +476,10 @@ __global__ void __launch_bounds__(kVmThreads, 1)
     __syncthreads();
     if (tl && threadIdx.x == 0)
         tl[5] = ptx::globaltimer_ns();
-    ptx::cluster_arrive_release();
+    if (*reinterpret_cast<volatile int32_t *>(&bars->abort))
+        ptx::cluster_arrive_release();
+    else
+        ptx::cluster_arrive_relaxed();
 #pragma unroll
     for (int i = 0; i < 2; ++i)
         if (pend_idx[i] >= 0) {
