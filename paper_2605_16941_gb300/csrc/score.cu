@@ -325,8 +325,8 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
                             break;
                         }
                         issue(acc0, sA(stage), sB(stage, 0), kb);
-                        if (kb == a.n_kb - 1)  // accumulator 0 is done: its epilogue need not wait for accumulator 1
-                            ptx::mma_commit_pair_multicast(tfull(acc0), kBothCtas);
+                        if (kTwo && kb == a.n_kb - 1)  // accumulator 0 is done: its epilogue need not wait for 1
+                            ptx::mma_commit_pair_multicast(tfull(0), kBothCtas);
                         if (kb < defer) {
                             if (kb == defer - 1) {  // the second accumulator is needed now
                                 if (!wait_acc_free(1, (uint32_t)item)) {
@@ -353,8 +353,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
                     }
                     if (aborted)
                         break;
-                    if (kTwo)  // the epilogue waits for both accumulators of every pass
-                        ptx::mma_commit_pair_multicast(tfull(1), kBothCtas);
+                    // The epilogue waits for both accumulators of every pass, or for the tile's one.  This commit is
+                    // the item's last: whoever has waited for it has the stage barriers' arrivals behind it as well.
+                    ptx::mma_commit_pair_multicast(tfull(kTwo ? 1 : acc0), kBothCtas);
                     tiles += two ? 2 : 1;
                     last_two = two;
                 }
@@ -492,7 +493,8 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
     __syncthreads();
     if (tl && threadIdx.x == 0)
         tl[5] = ptx::globaltimer_ns();
-    if (*reinterpret_cast<volatile int32_t *>(&bars->abort))
+    const bool gave_up = *reinterpret_cast<volatile int32_t *>(&bars->abort) != 0;
+    if (gave_up)
         ptx::cluster_arrive_release();
     else
         ptx::cluster_arrive_relaxed();
@@ -508,11 +510,13 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
         // status word, has completed: a failure recorded now belongs to this call.
         if (!tmem_ok)
             atomicExch(&a.status->current, (int32_t)WINO_ERR_UNSUPPORTED);
-        else if (*reinterpret_cast<volatile int32_t *>(&bars->abort))
+        else if (gave_up)
             atomicExch(&a.status->current, (int32_t)WINO_ERR_DEVICE_TIMEOUT);
     }
     ptx::cluster_wait_acquire();
     ptx::tc_fence_after();
+    if (gave_up)
+        settle_peer_arrivals();
     if (warp == 1)
         ptx::tmem_dealloc_pair(tmem, kTmemCols);
     if (tl && threadIdx.x == 0)

@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(kVmThreads, 1)
                         break;
                     }
                     issue(acc0, stage, it.h0, kb);
-                    if (kb == a.n_kb - 1)  // accumulator 0 is done: its epilogue need not wait for accumulator 1
+                    if (both && kb == a.n_kb - 1)  // accumulator 0 is done: its epilogue need not wait for 1
                         ptx::mma_commit_pair_multicast(tfull(acc0), kBothCtas);
                     if (second) {
                         if (both)
@@ -327,8 +327,8 @@ __global__ void __launch_bounds__(kVmThreads, 1)
                 }
                 if (aborted)
                     break;
-                if (both)
-                    ptx::mma_commit_pair_multicast(tfull(acc1), kBothCtas);
+                // the item's last commit (see score.cu)
+                ptx::mma_commit_pair_multicast(tfull(both ? acc1 : acc0), kBothCtas);
                 tiles += it.h0 == 0;
             }
             // No MMA may still be writing either CTA's TMEM when it is released.
@@ -471,12 +471,13 @@ __global__ void __launch_bounds__(kVmThreads, 1)
         }
     }
 
-    // Neither CTA releases TMEM, or exits, while its peer may still use the pair's TMEM or barriers.
+    // Neither CTA releases TMEM, or exits, while its peer may still use the pair's TMEM or barriers (see score.cu).
     ptx::tc_fence_before();
     __syncthreads();
     if (tl && threadIdx.x == 0)
         tl[5] = ptx::globaltimer_ns();
-    if (*reinterpret_cast<volatile int32_t *>(&bars->abort))
+    const bool gave_up = *reinterpret_cast<volatile int32_t *>(&bars->abort) != 0;
+    if (gave_up)
         ptx::cluster_arrive_release();
     else
         ptx::cluster_arrive_relaxed();
@@ -491,11 +492,13 @@ __global__ void __launch_bounds__(kVmThreads, 1)
         // Warp 2 has passed griddepcontrol.wait: a failure recorded now belongs to this call (see score.cu).
         if (!tmem_ok)
             atomicExch(&a.status->current, (int32_t)WINO_ERR_UNSUPPORTED);
-        else if (*reinterpret_cast<volatile int32_t *>(&bars->abort))
+        else if (gave_up)
             atomicExch(&a.status->current, (int32_t)WINO_ERR_DEVICE_TIMEOUT);
     }
     ptx::cluster_wait_acquire();
     ptx::tc_fence_after();
+    if (gave_up)
+        settle_peer_arrivals();
     if (warp == 1)
         ptx::tmem_dealloc_pair(tmem, kTmemCols);
     if (tl && threadIdx.x == 0)

@@ -15,6 +15,7 @@
 namespace wino {
 
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s per wait
+constexpr uint64_t kSettleNs = 100000ull;  // 0.1 ms, only after a wait gave up
 constexpr uint64_t kDrainLimitNs = 200000000ull;  // 0.2 s for draining after an abort
 
 // Wait for phase `parity` of `bar`; false once `limit_ns` passed (the abort flag is then raised) or another
@@ -48,6 +49,15 @@ __device__ inline bool wait_drain(uint32_t bar, uint32_t parity, uint64_t limit_
         if (ptx::globaltimer_ns() - t0 > limit_ns)
             return false;
     return true;
+}
+
+// After a wait gave up, a CTA no longer waits for the relaxed arrivals that its peer sent before the closing cluster
+// barrier: its barriers stay in place long enough for them to land (they take about a microsecond).
+__device__ inline void settle_peer_arrivals()
+{
+    const uint64_t t0 = ptx::globaltimer_ns();
+    while (ptx::globaltimer_ns() - t0 < kSettleNs) {
+    }
 }
 
 }  // namespace wino
