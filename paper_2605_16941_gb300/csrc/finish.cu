@@ -45,7 +45,6 @@ namespace {
 
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr int kFinishRows = 8;  // rows (warps) per finish_kernel CTA; also the CTA size of draft_verify_kernel
-constexpr int kClusterSeqRows = 256;  // rows of a sequence up to which a cluster of CTAs finishes it: two per warp
 constexpr int kRecInFlight = 5;  // records each lane loads at once (160 per row: two per pair of a 76-pair launch fit)
 
 // Block-wide reduction scratch for eq4_block.
@@ -601,7 +600,7 @@ cudaError_t launch_gather_active(const uint16_t *H, uint16_t *Hc, int32_t *targe
 cudaError_t launch_finish(FinishArgs a, cudaStream_t stream)
 {
     const wino_params &p = a.p;
-    a.seq_rows = a.tokens ? ((p.options & (WINO_OPT_NO_SHADOW | WINO_OPT_COMPACT)) ? 1 : 2) * p.blk_len : 0;
+    a.seq_rows = a.tokens ? (int32_t)rows_per_seq(p) : 0;
     const bool clusters = a.tokens && a.seq_rows <= kClusterSeqRows;
     const int warps = clusters && a.seq_rows > 128 ? 16 : kFinishRows;
     a.cluster = clusters ? std::min(8, (a.seq_rows + warps - 1) / warps) : 1;  // 8: the portable most

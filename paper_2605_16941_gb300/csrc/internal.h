@@ -61,6 +61,25 @@ constexpr uint32_t kVmRingCapacity = kScoreSmemMax - kVmSmemOverhead;
 
 constexpr int kMaxBlkLen = 1024;
 
+// Rows of a sequence up to which a cluster of CTAs ends a step (finish_step_kernel, which states why); longer
+// sequences hand their rows over through tickets (finish_kernel).
+constexpr int kClusterSeqRows = 256;
+
+// Rows that a step scores per sequence: block and shadow rows, or one row per position.
+inline int64_t rows_per_seq(const wino_params &p)
+{
+    return ((p.options & (WINO_OPT_NO_SHADOW | WINO_OPT_COMPACT)) ? 1 : 2) * (int64_t)p.blk_len;
+}
+
+// Tickets that the end of a step over N scored rows counts on: one per scored sequence (not per sequence of the batch,
+// of which an active-sequence list may name few), none where clusters end the step.  Fewer than N / 256, so the
+// ceil(N / 2) that a workspace reserves hold them.
+inline int32_t step_tickets(const wino_params &p, int64_t N)
+{
+    const int64_t rows = rows_per_seq(p);
+    return rows <= kClusterSeqRows ? 0 : (int32_t)(N / rows);
+}
+
 // Where a scored row's target token comes from.
 struct TargetSource {
     const int32_t *target;  // explicit per-row targets (wino_score_rows), or nullptr
@@ -155,7 +174,7 @@ struct FinishArgs {
     wino_params p;
     int32_t *counts;
     int8_t *flags;
-    int32_t *tickets;  // [n_seq], zero on entry
+    int32_t *tickets;  // [step_tickets], zero on entry
     // set by launch_finish
     int32_t seq_rows;  // rows of a sequence
     int32_t cluster;   // CTAs per sequence (finish_step_kernel)

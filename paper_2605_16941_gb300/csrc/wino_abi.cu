@@ -275,7 +275,9 @@ int score_and_finish(const uint16_t *H, const uint16_t *W, bool w_panels, int64_
     a.part_u = entropy ? reinterpret_cast<float *>(w8 + L.part_u) : nullptr;
     a.status = reinterpret_cast<StatusWords *>(w8 + L.status);
     a.tickets = reinterpret_cast<int32_t *>(w8 + L.tickets);
-    a.n_tickets = step ? step->n_seq : 0;
+    a.n_tickets = step ? step_tickets(*step, N) : 0;
+    if ((size_t)a.n_tickets * 4 > L.part - L.tickets)
+        return WINO_ERR_WORKSPACE;  // the score kernel clears that many
     a.timeline = timeline_slot((unsigned)(2 * a.n_groups * a.G));
     a.w_panels = w_panels ? 1 : 0;
     prof_record(0, stream);
@@ -310,8 +312,7 @@ int score_and_finish(const uint16_t *H, const uint16_t *W, bool w_panels, int64_
 // Rows wino_step scores for these parameters, and the workspace it needs.
 int64_t step_rows(const wino_params &p)
 {
-    const bool one_row = (p.options & (WINO_OPT_NO_SHADOW | WINO_OPT_COMPACT)) != 0;
-    return (int64_t)(p.active_seq ? p.n_active : p.n_seq) * (one_row ? 1 : 2) * p.blk_len;
+    return (int64_t)(p.active_seq ? p.n_active : p.n_seq) * rows_per_seq(p);
 }
 
 size_t step_ws_bytes(const wino_params &p, int64_t d, int64_t V)
