@@ -531,10 +531,8 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
 // per-pass overhead, the widest tile, fewest passes over W (more groups).  A width below kBN pays when the
 // vocabulary then splits evenly over the pairs: V = 126464 on 76 pairs is 494 tiles of 256 (7 on the
 // busiest pair, 6.5 on average) but 527 tiles of 240 (7 on 71 pairs).
-#ifndef WINO_PASS_MIN_ROW_BLOCKS
-#define WINO_PASS_MIN_ROW_BLOCKS 2  // compile-time tuning: fewest 256-row blocks that use passes
-#endif
-constexpr int32_t kPassMinRowBlocks = WINO_PASS_MIN_ROW_BLOCKS;
+constexpr int32_t kPassMinRowBlocks = 2;  // fewest 256-row blocks that use passes
+static_assert(kPassMinRowBlocks <= 2, "single tiles merge their row states in the ring, which is free after one sweep only");
 
 ScoreSchedule score_schedule(int32_t n_mb, int64_t V, int max_units, int32_t records_cap)
 {
@@ -638,6 +636,8 @@ cudaError_t launch_score(const CUtensorMap &tmH, const CUtensorMap &tmW, const S
     // The ring must hold what the producer stages: a pass's third slot takes an H box (16 KB) in a row-pair
     // sweep, which the launch has when a group owns more than one row block.
     const uint32_t wb = stage_bytes_w(a.bn);
+    if (!a.two && a.n_mb > a.n_groups)
+        return cudaErrorInvalidValue;  // a second sweep's copies would run into the merge scratch
     const uint32_t merge = a.two ? kMergeBytes : 0u;
     const uint32_t third = a.two ? (a.n_mb > a.n_groups && wb < kStageBytesA ? kStageBytesA : wb) : 0u;
     if (a.stages < 2 || a.stages > kMaxStages || a.stage_bytes < kStageBytesA + wb + third ||

@@ -60,6 +60,14 @@ def test_split_invariants(sm, pairs):
         assert wino.wino_workspace_size(N, 4096, V) >= N * p["G"] * 16
 
 
+@pytest.mark.parametrize("sm,pairs", DEVICES, ids=[f"sm{a}_p{b}" for a, b in DEVICES])
+def test_single_tiles_have_one_sweep(sm, pairs):
+    """Single tiles merge their row states in the ring at the end of a sweep, so no group may own two row blocks."""
+    for N, V in itertools.product([*ROWS, 511, 513, 768], VOCABS):
+        p = wino.wino_score_plan_host(N, 4096, V, sm, pairs)
+        assert p["two"] or p["n_mb"] <= p["n_groups"], p
+
+
 def _walk(plan):
     """The items each CTA pair computes, in the order the score kernel's three roles walk them: per pair a
     list of items, each a list of (row block, tile, accumulator); and the vocabulary sweeps per group."""
