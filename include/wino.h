@@ -356,7 +356,8 @@ WINO_API int wino_profile_end(double *score_ms_total, int *score_launches);
  * come from one thread and are ordered; [3] and [4] come from other warps,
  * whose %globaltimer readings were seen to disagree with it by up to a few
  * microseconds, so compare those only with each other or across CTAs.
- * A launch with more CTAs than ctas_per_launch writes nothing.  buf is a
+ * A launch with more CTAs than ctas_per_launch (wino_score_launch tells a
+ * launch's) writes nothing.  buf is a
  * device buffer of n_launches * ctas_per_launch * 8 uint64 owned by the
  * caller; end returns how many launches were counted.  One timeline per
  * process at a time.
@@ -368,7 +369,8 @@ WINO_API int wino_timeline_end(int64_t *launches);
  * How the row-block score kernel splits a launch of N rows over V entries on
  * the current device (diagnostics; the paper has no counterpart).  Row counts
  * that do not fill 256-row blocks mostly run on the vocabulary-major kernel
- * instead, whose split this call does not describe.  plan (host int32[8]) receives
+ * instead; wino_score_launch tells which kernel runs and describes either
+ * split.  plan (host int32[8]) receives
  * the tile width bn, the vocabulary tiles n_vt = ceil(V / bn), the 256-row
  * blocks n_mb, the row-block groups, the CTA pairs per group G (= records per
  * row), the grid size in CTAs, 1 if the kernel works in passes (each staged
@@ -389,6 +391,26 @@ WINO_API int wino_score_plan(int64_t N, int64_t d, int64_t V, int32_t *plan);
  */
 WINO_API int wino_score_plan_host(int64_t N, int64_t d, int64_t V, int32_t sm_count, int32_t max_pairs,
                                   int32_t *plan);
+
+/*
+ * Which score kernel wino_score_rows and wino_step run for N scored rows of
+ * width d over V entries, and how it splits the launch, on a device with
+ * sm_count SMs and max_pairs resident pairs, or with both 0 on the current
+ * device (diagnostics: timelines, capacity planning, host-side tests).
+ * launch (host int32[14]) receives [0] the kernel: 0 row blocks in single
+ * tiles, 1 row blocks in passes, 2 vocabulary-major; [1] the tile width bn;
+ * [2] the vocabulary tiles n_vt; [3] the groups of CTA pairs (each owns the
+ * row blocks of wino_score_plan, or of the vocabulary-major kernel one block
+ * of hw0 + hw1 rows); [4] the pairs per group G; [5] the grid size in CTAs;
+ * [6] the partial records per row; [7] the ring stages and [8] the bytes of
+ * one; [9] a CTA's dynamic shared memory in bytes; and, 0 unless the kernel is
+ * 2, [10] hw0 and [11] hw1, the rows of the one or two accumulators of a tile
+ * (hw1 = 0: one), [12] the accumulators held in tensor memory, [13] 1 if the
+ * last round's tiles are shared by two pairs, one accumulator each.  Pair c
+ * belongs to group c % groups and computes tiles c / groups (+ G, ...).
+ */
+WINO_API int wino_score_launch(int64_t N, int64_t d, int64_t V, int32_t sm_count, int32_t max_pairs,
+                               int32_t *launch);
 
 /*
  * Self-test of the failure path (device-side timeout handling; the paper has

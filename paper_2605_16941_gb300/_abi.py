@@ -35,7 +35,7 @@ WINO_OPT_W_PANELS = 8
 EXPORTS = ("wino_workspace_size", "wino_workspace_size_step", "wino_score_rows", "wino_draft_verify", "wino_step",
            "wino_step_static_scratch", "wino_read_device_status", "wino_profile_begin", "wino_profile_end",
            "wino_selftest_wait_timeout", "wino_status_string", "wino_version", "wino_decode", "wino_timeline_begin",
-           "wino_timeline_end", "wino_score_plan", "wino_score_plan_host", "wino_lm_head_panels")
+           "wino_timeline_end", "wino_score_plan", "wino_score_plan_host", "wino_score_launch", "wino_lm_head_panels")
 
 # 64-bit words per CTA in a score-kernel timeline (wino_timeline_begin)
 TIMELINE_WORDS = 8
@@ -101,6 +101,8 @@ def lib() -> C.CDLL:
         L.wino_profile_end.argtypes = [C.POINTER(C.c_double), C.POINTER(C.c_int)]
         L.wino_score_plan_host.restype = C.c_int
         L.wino_score_plan_host.argtypes = [i64, i64, i64, C.c_int32, C.c_int32, C.POINTER(C.c_int32)]
+        L.wino_score_launch.restype = C.c_int
+        L.wino_score_launch.argtypes = [i64, i64, i64, C.c_int32, C.c_int32, C.POINTER(C.c_int32)]
         L.wino_score_plan.restype = C.c_int
         L.wino_score_plan.argtypes = [i64, i64, i64, C.POINTER(C.c_int32)]
         L.wino_timeline_begin.restype = C.c_int
@@ -332,6 +334,15 @@ def wino_score_plan_host(N: int, d: int, V: int, sm_count: int = 152, max_pairs:
            "wino_score_plan_host")
     return dict(zip(("bn", "n_vt", "n_mb", "n_groups", "G", "ctas", "two", "stages", "stage_bytes",
                      "records_per_row"), list(out)))
+
+
+def wino_score_launch(N: int, d: int, V: int, sm_count: int = 0, max_pairs: int = 0) -> dict:
+    """The score kernel that runs for N rows (``kernel``: 0 row blocks in single tiles, 1 row blocks in passes,
+    2 vocabulary-major) and its work split, on the current device or a described one."""
+    out = (C.c_int32 * 14)()
+    _check(lib().wino_score_launch(int(N), int(d), int(V), int(sm_count), int(max_pairs), out), "wino_score_launch")
+    return dict(zip(("kernel", "bn", "n_vt", "n_groups", "G", "ctas", "records", "stages", "stage_bytes", "smem_bytes",
+                     "hw0", "hw1", "slots", "split"), list(out)))
 
 
 def wino_timeline_begin(buf, n_launches: int, ctas_per_launch: int) -> None:

@@ -212,6 +212,10 @@ inline int64_t records_per_row(int64_t V)
 // CTA pairs of the score kernel that can be resident at once on the current device (<= 0 on error).
 int score_max_pairs();
 
+// Dynamic shared memory of a score CTA with a ring of `ring` bytes: row-block kernel, vocabulary-major kernel.
+constexpr uint32_t score_smem_bytes(bool two, uint32_t ring) { return kSmemOverhead + (two ? kMergeBytes : 0u) + ring; }
+constexpr uint32_t vmajor_smem_bytes(uint32_t ring) { return kVmSmemOverhead + ring; }
+
 // entropy: also accumulate part_u (the variant used when wino_score_rows is asked for H(p)).
 cudaError_t launch_score(const CUtensorMap &tmH, const CUtensorMap &tmW, const ScoreArgs &a, bool entropy,
                          cudaStream_t stream);

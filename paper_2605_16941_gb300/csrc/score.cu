@@ -638,7 +638,6 @@ cudaError_t launch_score(const CUtensorMap &tmH, const CUtensorMap &tmW, const S
     const uint32_t wb = stage_bytes_w(a.bn);
     if (!a.two && a.n_mb > a.n_groups)
         return cudaErrorInvalidValue;  // a second sweep's copies would run into the merge scratch
-    const uint32_t merge = a.two ? kMergeBytes : 0u;
     const uint32_t third = a.two ? (a.n_mb > a.n_groups && wb < kStageBytesA ? kStageBytesA : wb) : 0u;
     if (a.stages < 2 || a.stages > kMaxStages || a.stage_bytes < kStageBytesA + wb + third ||
         a.stage_bytes % 1024u != 0 || (uint64_t)a.stages * a.stage_bytes > (a.two ? kPassRingCapacity : kRingCapacity) ||
@@ -646,7 +645,8 @@ cudaError_t launch_score(const CUtensorMap &tmH, const CUtensorMap &tmW, const S
         return cudaErrorInvalidValue;
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = score_launch_config((unsigned)(2 * a.n_groups * a.G), kScoreThreads,
-                                                 kSmemOverhead + merge + (uint32_t)a.stages * a.stage_bytes, stream, attr);
+                                                 score_smem_bytes(a.two != 0, (uint32_t)a.stages * a.stage_bytes), stream,
+                                                 attr);
     if (entropy)
         return a.two ? cudaLaunchKernelEx(&cfg, score_kernel<true, true>, tmH, tmW, a)
                      : cudaLaunchKernelEx(&cfg, score_kernel<true, false>, tmH, tmW, a);

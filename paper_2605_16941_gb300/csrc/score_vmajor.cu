@@ -614,7 +614,7 @@ cudaError_t launch_score_vmajor(const CUtensorMap &tmH, const CUtensorMap &tmW, 
         return cudaErrorInvalidValue;
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = score_launch_config((unsigned)(2 * a.n_groups * a.G), kVmThreads,
-                                                 kVmSmemOverhead + (uint32_t)ring, stream, attr);
+                                                 vmajor_smem_bytes((uint32_t)ring), stream, attr);
     return entropy ? cudaLaunchKernelEx(&cfg, score_vmajor_kernel<true>, tmH, tmW, a)
                    : cudaLaunchKernelEx(&cfg, score_vmajor_kernel<false>, tmH, tmW, a);
 }

@@ -214,6 +214,36 @@ int check_params(const wino_params *p)
     return WINO_OK;
 }
 
+// Which score kernel takes a launch, and its split: `sch`, for the vocabulary-major kernel with that kernel's tiles,
+// groups and ring in place of the row-block kernel's, and `vm` for what only that kernel has.
+struct ScoreLaunch {
+    ScoreSchedule sch;
+    VmSchedule vm;
+    bool vmajor;
+    int32_t records;  // records per row: one per pair, one per CTA from the vocabulary-major kernel
+    uint32_t ctas() const { return (uint32_t)(2 * sch.n_groups * sch.G); }
+};
+
+ScoreLaunch plan_launch(int64_t N, int64_t d, int64_t V, int units)
+{
+    const int32_t cap = (int32_t)records_per_row(V);
+    ScoreLaunch l{};
+    l.sch = score_schedule((int32_t)((N + kPairM - 1) / kPairM), V, units, cap);
+    l.vmajor = score_vmajor_schedule(N, d, V, units, cap, l.sch, &l.vm);
+    if (l.vmajor) {
+        l.sch.bn = l.vm.bn;
+        l.sch.n_vt = l.vm.n_vt;
+        l.sch.n_groups = l.vm.n_groups;
+        l.sch.G = l.vm.G;
+        l.sch.stages = l.vm.stages;
+        l.sch.stage_bytes = l.vm.stage_bytes;
+    } else {
+        l.vm = VmSchedule{};
+    }
+    l.records = l.vmajor ? 2 * l.sch.G : l.sch.G;
+    return l;
+}
+
 // Score N rows into (argmax, pmax, ptarget), and with `step` also apply Eq. 4:
 // the score kernel followed by the finish kernel.
 // W is row-major [V, d], or with w_panels the panel copy [d/64][V][64] of wino_lm_head_panels.
@@ -233,18 +263,10 @@ int score_and_finish(const uint16_t *H, const uint16_t *W, bool w_panels, int64_
     if (max_pairs < 1)
         return WINO_ERR_CUDA;
     const int32_t n_mb = (int32_t)((N + kPairM - 1) / kPairM);
-    const int units = std::min(max_pairs, info.sm_count / 2);
-    ScoreSchedule sch = score_schedule(n_mb, V, units, (int32_t)records_per_row(V));
-    VmSchedule vm{};
-    const bool vmajor = score_vmajor_schedule(N, d, V, units, (int32_t)records_per_row(V), sch, &vm);
-    if (vmajor) {
-        sch.bn = vm.bn;
-        sch.n_vt = vm.n_vt;
-        sch.n_groups = vm.n_groups;
-        sch.G = vm.G;
-        sch.stages = vm.stages;
-        sch.stage_bytes = vm.stage_bytes;
-    }
+    const ScoreLaunch launch = plan_launch(N, d, V, std::min(max_pairs, info.sm_count / 2));
+    const ScoreSchedule &sch = launch.sch;
+    const VmSchedule &vm = launch.vm;
+    const bool vmajor = launch.vmajor;
     CUtensorMap tmH, tmW;
     if ((rc = tensor_map(H, N, d, vmajor ? (vm.hw[0] + vm.hw[1]) / 2 : kBM, &tmH)) != WINO_OK)
         return rc;
@@ -278,7 +300,7 @@ int score_and_finish(const uint16_t *H, const uint16_t *W, bool w_panels, int64_
     a.n_tickets = step ? step_tickets(*step, N) : 0;
     if ((size_t)a.n_tickets * 4 > L.part - L.tickets)
         return WINO_ERR_WORKSPACE;  // the score kernel clears that many
-    a.timeline = timeline_slot((unsigned)(2 * a.n_groups * a.G));
+    a.timeline = timeline_slot(launch.ctas());
     a.w_panels = w_panels ? 1 : 0;
     prof_record(0, stream);
     if ((vmajor ? launch_score_vmajor(tmH, tmW, a, entropy != nullptr, stream)
@@ -289,7 +311,7 @@ int score_and_finish(const uint16_t *H, const uint16_t *W, bool w_panels, int64_
     f.part = a.part;
     f.part_u = a.part_u;
     f.entropy = entropy;
-    f.G = vmajor ? 2 * a.G : a.G;  // one record per CTA of a pair from the vocabulary-major kernel
+    f.G = launch.records;
     f.N = a.N;
     f.V = a.V;
     f.ts = ts;
@@ -604,6 +626,41 @@ int wino_score_plan(int64_t N, int64_t d, int64_t V, int32_t *plan)
     plan[5] = 2 * sch.n_groups * sch.G;
     plan[6] = sch.two;
     plan[7] = sch.stages;
+    return WINO_OK;
+}
+
+int wino_score_launch(int64_t N, int64_t d, int64_t V, int32_t sm_count, int32_t max_pairs, int32_t *launch)
+{
+    const bool current = sm_count == 0 && max_pairs == 0;
+    if (!launch || (!current && (sm_count < 2 || max_pairs < 1)))
+        return WINO_ERR_ARG;
+    if (!shape_ok(N, d, V))
+        return WINO_ERR_SHAPE;
+    if (current) {
+        DeviceInfo info;
+        int rc = device_info(&info);
+        if (rc != WINO_OK)
+            return rc;
+        sm_count = info.sm_count;
+        if ((max_pairs = score_max_pairs()) < 1)
+            return WINO_ERR_CUDA;
+    }
+    const ScoreLaunch l = plan_launch(N, d, V, std::min(max_pairs, sm_count / 2));
+    const uint32_t ring = (uint32_t)l.sch.stages * l.sch.stage_bytes;
+    launch[0] = l.vmajor ? 2 : l.sch.two;
+    launch[1] = l.sch.bn;
+    launch[2] = l.sch.n_vt;
+    launch[3] = l.sch.n_groups;
+    launch[4] = l.sch.G;
+    launch[5] = (int32_t)l.ctas();
+    launch[6] = l.records;
+    launch[7] = l.sch.stages;
+    launch[8] = (int32_t)l.sch.stage_bytes;
+    launch[9] = (int32_t)(l.vmajor ? vmajor_smem_bytes(ring) : score_smem_bytes(l.sch.two != 0, ring));
+    launch[10] = l.vm.hw[0];
+    launch[11] = l.vm.hw[1];
+    launch[12] = l.vm.slots;
+    launch[13] = l.vm.split;
     return WINO_OK;
 }
 

@@ -90,7 +90,7 @@ def test_step_with_panels_is_bit_identical(name):
     _assert_same(a, b)
     c, e = _step_pair(w, H, Wd, Wp, st, compact=True)  # gathered rows: a different H, the same W path
     _assert_same(c, e)
-    print(name, "N", w.N, "plan", wino.wino_score_plan(w.N, w.d, w.V))
+    print(name, "N", w.N, "launch", wino.wino_score_launch(w.N, w.d, w.V))
 
 
 def test_static_scratch_and_library_loop_with_panels():
