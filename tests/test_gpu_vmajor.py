@@ -1,7 +1,8 @@
 """The vocabulary-major score kernel (csrc/score_vmajor.cu) against the fp64 oracle, at the edges of its row counts:
 one row, partial 32-row chunks, one accumulator of 32-multiple and of 16-multiple width, two accumulators of unequal
 and of equal width, several row groups with a ragged last one; vocabulary and K tails; with and without entropy.
-The launch's timeline shows that this kernel ran: its tile counts are not those of the row-block split."""
+The launch's timeline shows its tiles, and wino_score_launch that this kernel takes it (the tile counts of the first three
+shapes are those of the row-block split too, the others' are not)."""
 import math
 
 import numpy as np
@@ -18,6 +19,7 @@ SHAPES = [
     (1, 8, 19456, 1 * 76),         # one row, one K slice (mostly zero fill), one 32-column chunk
     (33, 72, 20001, 1 * 139),      # 64 columns, K tail, 144-wide tiles, the last one mostly past the vocabulary
     (48, 256, 40000, 1 * 228),     # 176-wide tiles
+    (40, 136, 47502, 1 * 213),     # 224-wide tiles
     (257, 512, 19456, 2 * 76),     # two groups of one accumulator of 144 columns (a half chunk at its end)
     (392, 512, 19456, 2 * 76),     # 208 columns
     (482, 512, 19456, 2 * 76),     # 256 columns
@@ -49,7 +51,10 @@ def _tiles(H, W, N, d, V):
 
 @pytest.mark.parametrize("N,d,V,tiles", SHAPES, ids=[f"N{s[0]}_d{s[1]}_V{s[2]}" for s in SHAPES])
 def test_matches_oracle(N, d, V, tiles):
+    import paper_2605_16941_gb300 as wino
     from gpu_helpers import compare_rows, dev, gpu_score
+    plan = wino.wino_score_launch(N, d, V)
+    assert plan["kernel"] == 2 and plan["n_groups"] * plan["n_vt"] == tiles
     H = ws.random_bf16(N, d, 1.0, seed=N * 5 + d)
     W = ws.random_bf16(V, d, 1.0 / math.sqrt(d), seed=V + d)
     rng = np.random.default_rng(N + V)
