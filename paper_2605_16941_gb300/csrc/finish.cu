@@ -54,8 +54,8 @@ struct Eq4Smem {
     float f0[kWarps];
 };
 
-// Dynamic shared memory of a launch with fixed-M drafting: pmax of each masked position, -inf elsewhere.  (Static, it
-// would keep the CTA from fitting beside a score CTA, see kScoreSmemMax.)
+// Dynamic shared memory of a launch with fixed-M drafting: pmax of each masked position, -inf elsewhere.  (Static, every
+// finish CTA would take its 4 KB and fewer would fit beside a score CTA, see kScoreSmemMax.)
 extern __shared__ float s_conf[];
 inline uint32_t conf_bytes(const wino_params &p) { return p.draft_m > 0 ? (uint32_t)p.blk_len * 4u : 0u; }
 
@@ -363,9 +363,13 @@ __device__ __forceinline__ void publish_status(const FinishArgs &a, int32_t stat
 // The end of a step whose sequences have at most kClusterSeqRows rows: a cluster of up to 8 CTAs per sequence.  Its
 // warps merge the sequence's rows and hand the statistics to the first CTA's shared memory; behind one cluster barrier
 // that CTA applies Eq. 4, whose tokens it has loaded meanwhile.
-// What bounds it is latency: dependent round trips to L2 and barriers after the score kernel's last CTA.  The CTAs are
-// small enough in registers and shared memory to start beside most score CTAs and wait there (with 64 registers and
-// 4.3 KB of shared memory they started only when score CTAs left: 9.5 -> 8.5 us for the tiny step in a CUDA graph).
+// What bounds it is latency: dependent round trips to L2 and barriers after the score kernel's last CTA.  The 8-warp CTAs
+// are small enough to start beside the row-block kernel's and wait there: 9.5 -> 8.5 us for the tiny step in a CUDA graph
+// against 64 registers and 4.3 KB of shared memory, both changed at once.  The 48 registers cost spills (36 bytes with 8
+// warps, 28 with 16); a step in a graph with 48 / 56 (12 and 24 bytes) / 64 (none): 6.60 / 6.77 / 6.43 us (d = 64, V = 1000, N = 64),
+// 12.43 / 12.58 / 12.13 (d = 512, V = 32000, N = 128).  Beside the vocabulary-major kernel the CTAs do not fit (168
+// registers a thread there); with 160 there they do, and nothing is gained: 149.4 -> 149.5 us (64 rows), 226.8 -> 227.3
+// (300), 25.4 -> 25.4 (333 rows, d = 1024, V = 32000, where finish_kernel follows).
 // Handing over through global memory (finish_kernel: one CTA per 8 rows, fences, a ticket per sequence, the statistics
 // read back) costs about 3 us more, but merges more rows at once.  us per step, finish_kernel -> here: 64 rows 9.2 ->
 // 7.9 (d = 64, V = 1000), 151.0 -> 147.8 (d = 4096, V = 126464); 128 rows 9.3 -> 8.5.  Above 128 rows with 16 warps per

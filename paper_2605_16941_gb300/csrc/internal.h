@@ -38,7 +38,11 @@ constexpr int kScoreThreads = 64 + 32 * kEpiWarps;  // warp 0 TMA, warp 1 TMEM +
 constexpr uint32_t kMergeBytes = (kEpiPerQuarter - 1) * 2 * kBM * 20;  // row states handed over at the end of a sweep
 constexpr uint32_t kStageBytesA = kBM * kBK * 2;  // 16 KB of H per stage
 constexpr uint32_t kSmemLimit = 227u * 1024u;  // the most dynamic shared memory a CTA may have
-// What a score CTA takes at most (a few pass-mode widths excepted), so that a finish CTA (1 KB reserved + 256 B static) fits beside it in an SM's 228 KB.
+// What a score CTA takes at most (a few pass-mode widths excepted), so that the shared memory of a finish_kernel CTA (1 KB
+// reserved + 176 B) fits beside it in an SM's 228 KB.  A finish_step_kernel CTA of 8 warps takes 1 KB + 128 B + 12 B per row
+// of a sequence: beside single tiles it fits up to 53 rows at the widest tile and up to 650 at the benchmark's (bn = 240).
+// Registers: 12 288 of an SM's 65 536 for 8 warps at 48, which the row-block kernel leaves (at most 144 x 320) and the
+// vocabulary-major kernel does not (168 x 320).
 constexpr uint32_t kScoreSmemMax = kSmemLimit - 1280u;
 constexpr uint32_t kSmemOverhead = 1024 /* ring alignment slack */ + 256 /* barriers */;
 constexpr uint32_t kRingCapacity = kScoreSmemMax - kSmemOverhead;

@@ -47,8 +47,8 @@
 //           know that the operands of tcgen05.mma, tcgen05.commit and the
 //           copies are warp-uniform, and issuing a K slice's MMAs then took
 //           longer than the MMAs themselves.  Branch on the lane index and a
-//           shuffle per wait, then elect.sync (us per step, 20-step regions at
-//           full clock; d = 4096, V = 126464): N = 64 168 -> 156, N = 256
+//           shuffle per wait, then elect.sync (us per step, 20-step regions;
+//           d = 4096, V = 126464): N = 64 168 -> 156, N = 256
 //           179 -> 166, N = 2048 1092 -> 1070; d = 1024, V = 64000, N = 2048
 //           247 -> 201;
 //   warps 2-9 epilogue (both CTAs): two warps per TMEM lane quarter, on the
@@ -354,7 +354,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
                     if (aborted)
                         break;
                     // The epilogue waits for both accumulators of every pass, or for the tile's one.  This commit is
-                    // the item's last: whoever has waited for it has the stage barriers' arrivals behind it as well.
+                    // the item's last: whoever has waited for it has the stage barriers' arrivals behind it as well,
+                    // assuming that the arrivals of one thread's successive commits reach a CTA in their order (PTX
+                    // states that each follows the MMAs issued before its commit, not an order among them).
                     ptx::mma_commit_pair_multicast(tfull(kTwo ? 1 : acc0), kBothCtas);
                     tiles += two ? 2 : 1;
                     last_two = two;
@@ -487,7 +489,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
 
     // Neither CTA releases TMEM, or exits, while its peer may still use the pair's TMEM or barriers.  No memory access
     // needs ordering by this barrier unless a wait gave up: every arrival sent to the leader's barriers has been
-    // waited for.  The release it then does without held every launch's end: us per step in a CUDA graph 6.9 -> 6.6
+    // waited for (for the peer's stage barriers see the item's last commit).  The release it then does without held every launch's end: us per step in a CUDA graph 6.9 -> 6.6
     // (d = 64, V = 1000, N = 64), 13.05 -> 12.56 (d = 512, V = 32000, N = 128).
     ptx::tc_fence_before();
     __syncthreads();

@@ -38,25 +38,28 @@ constexpr int kVmEpiWarps = 8;
 constexpr int kVmThreads = 64 + 32 * kVmEpiWarps;
 constexpr int kMaxChunks = 4;  // 32-column chunks of one accumulator (256 columns) per epilogue warp
 
-// The split and the choice between the two score kernels: ns on the busiest pair, fitted to calls of both kernels (123
-// and 49 of this one with one and two accumulators per tile, 34 of score.cu, at d = 256 to 2560, rms 5 %, and the
-// d = 4096 rows below).  Per tile and K slice, from 24 K slices on (long enough for the board's power limit) and below:
+// The split and the choice between the two score kernels: estimated ns on the busiest pair, fitted to measured calls of
+// both.  Per tile and K slice, from 24 K slices on (long enough for the board's power limit) and below:
 //   one accumulator    190 + 0.75 hw,                   204 + 0.22 hw;
 //   two                60 + 1.4 w and 4 w per tile,     1.25 w - 12 and 8 w per tile, w = hw[0] + hw[1];
 //   score.cu           0.95 (bn + 144) and 700 per tile, 1.75 (bn - 55) and 607 per tile;
 // here the epilogue (540 for two 32-column chunks, one per warp of a quarter) if that is longer, plus a third of the
 // shorter of the two for one accumulator below 24 K slices; and the last tile's epilogue.
-// us per step, score.cu -> here (groups), d = 4096, V = 126464: N = 288 308 -> 209 (1), 320 316 -> 238 (1),
-// 384 326 -> 271 (1), 448 333 -> 312 (2), 512 344 -> 346 (2), 576 494 -> 390 (2), 640 502 -> 421 (2), 768 523 -> 482 (3),
-// 896 616 -> 578 (4), 1024 632 -> 620 (4), 1280 870 -> 771 (5), 1664 1171 -> 1036 (4), 2048 1204 -> 1213 (stays with
-// score.cu); d = 1664, V = 64677: 310 71.1 -> 53.0 (1); d = 576, V = 103363: 308 48.6 -> 37.4 (2); d = 512, V = 54379:
-// 1298 67.5 -> 59.9 (6); d = 448, V = 54533: 373 27.1 -> 23.9 (2); d = 256, V = 64000: 384 19.4 -> 25.6 (3; stays).
-// On those 34 calls the choice was on average within 1 % of the best split of either kernel and at most 1.4 % slower than
-// score.cu; on 36 others that it sent here 7 % faster on average and at most 4 % slower.
+// us per call of wino_score_rows, score.cu -> here (groups), both on the same inputs in turn, d = 4096, V = 126464:
+// N = 288 275 -> 202 (1), 320 285 -> 221 (1), 384 292 -> 272 (1), 448 297 -> 284 (2), 512 303 -> 313 (2), 576 465 -> 373 (2),
+// 640 471 -> 422 (2), 768 483 -> 459 (3), 896 570 -> 549 (4), 1024 576 -> 598 (4), 1280 815 -> 775 (5), 1664 1177 -> 1068 (4),
+// 2048 1214 -> 1198 (8; stays with score.cu); d = 1664, V = 64677: 310 67.3 -> 54.7 (1); d = 576, V = 103363: 308 48.8 ->
+// 36.7 (2); d = 512, V = 54379: 1298 66.1 -> 59.5 (6); d = 448, V = 54533: 373 24.5 -> 23.9 (2); d = 256, V = 64000: 384 18.9 ->
+// 24.7 (2; stays).
+// Of 48 random shapes (N = 49 to 2048, d = 320 to 4096, V = 19456 to 134400) the choice sent 29 here, all with more than
+// 256 rows: 0.90 of score.cu's time (geometric mean; 0.77 at N = 304, d = 2112, V = 121643 to 1.06 at N = 907, d = 448,
+// V = 65313), six of them 1.6 to 6.3 % slower than score.cu, and 1.01 of the best split's of either kernel.
 // Up to 256 rows (one row block) both kernels follow the W stream.  This one wins where score.cu's mostly
-// empty boxes of H hold it up (N = 32, d = 1024 38.0 -> 30.4; N = 64 30.2 -> 30.9) and where the W stream is long
-// enough for the power limit to bite (d = 3072, V = 126464, N = 128 129 -> 119; d = 4096 168 -> 154, N = 208 175 -> 171,
-// N = 256 183 -> 190; but d = 2048, V = 64000, N = 128 49.6 -> 50.3).
+// empty boxes of H hold it up (N = 32, d = 1024 33.8 -> 26.6; N = 64 27.0 -> 27.6) and where the W stream is long
+// enough for the power limit to bite (N = 128: d = 3072, V = 126464 124.7 -> 123.0; d = 4096 163.8 -> 159.0; but d = 4096,
+// N = 208 177.4 -> 183.6, and d = 2048, V = 64000, N = 128 48.0 -> 48.4).  Of the 14 random shapes of 49 to 256 rows, all with
+// score.cu, five would have been 12 to 32 % faster here (49 to 112 rows, d = 576 to 960): the line at
+// kVmShortRows lies low for such heads.
 constexpr int kVmCappedSlices = 24;
 constexpr int kVmShortRows = 48;                        // always here (with a vocabulary for every pair's records)
 constexpr int kVmMinSlices = 5;                         // K slices per tile: below, latencies that the estimates leave out
@@ -82,7 +85,7 @@ static_assert(sizeof(VmBarriers) <= kVmBarrierBytes, "barrier block must fit its
 // Item i of the pair at column `col` of its group: vocabulary tile vt, accumulators [h0, h1).  Rounds of whole tiles
 // col, col + G, ...; in a last round that would leave at least half of the pairs idle (ScoreArgs::split), a tile's two
 // accumulators go to two pairs (V = 126464 on 76 pairs: 6.5 tiles a pair instead of 7; us per step at d = 4096, N = 288
-// 215.5 -> 209.5, 300 222.5 -> 217.5, 384 275.3 -> 270.3, steady state; 352 at full clock 229 -> 219).
+// 215.5 -> 209.5, 300 222.5 -> 217.5, 384 275.3 -> 270.3, steady state; 352 in 20-step regions 229 -> 219).
 struct VmItem {
     int vt, h0, h1;
 };

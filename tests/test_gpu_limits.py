@@ -71,7 +71,7 @@ def test_score_rows_max_dimension():
 
 
 def test_step_many_sequences():
-    """One step over 4096 sequences with blocks of 4 (N = 32 768 rows, 4096 Eq. 4 tickets) against the
+    """One step over 4096 sequences with blocks of 4 (N = 32 768 rows, each sequence ended by a CTA of its own) against the
     whole oracle step."""
     import paper_2605_16941_gb300 as wino
     from gpu_helpers import compare_step, dev, host
